@@ -92,10 +92,12 @@ typedef enum {
                                 FP32 arithmetic only; where a plane's rows do not fit in shared
                                 memory the compact two-pass update runs instead (see
                                 lbm_resolved_kernel) */
-    LBM_KERNEL_PERSISTENT = 6  /* the compact two-pass update, n updates in one cooperative launch
-                                with grid-wide barriers between the passes (for small instances
-                                and batches of them); no wall slip; a barrier
-                                that waits about two seconds gives up, and the next
+    LBM_KERNEL_PERSISTENT = 6  /* the compact two-pass update, n updates in one launch (for small
+                                instances and batches of them); no wall slip.  FP32 and 16-bit
+                                storages whose instances have at most 8192 non-solid cells keep
+                                each instance in the shared memory of one thread-block cluster;
+                                otherwise one cooperative launch with grid-wide barriers between
+                                the passes, of which a barrier that waits about two seconds gives up, and the next
                                 lbm_reduce, lbm_get_fields or lbm_run_to_steady returns
                                 LBM_ERR_TIMEOUT */
 } lbm_kernel;

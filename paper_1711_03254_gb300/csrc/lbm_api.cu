@@ -67,6 +67,7 @@ struct lbm_ctx {
     bool persist_used = false; // a persistent launch ran since the flag was last read
     long long bar_cycles = 4000000000LL;  // bound on a barrier wait (about 2 s of SM clock)
     unsigned bar_missing = 0;  // failure test: arrivals the barriers wait for that never come
+    int onchip = 0;  // threads per block of the on-chip persistent update (0: does not fit)
     FcPlan fplan{};  // single-read fused update on the compact layout (ok when it fits)
     std::vector<uint32_t> plane_start;  // compact index of each plane's first cell (instance 0), nz + 1
     bool half_step = false;             // the density pass of a split update has run
@@ -228,13 +229,19 @@ lbm_kernel resolve_kernel(const lbm_ctx *ctx, int n) {
     // memory; where they do not, its layout's two-pass update runs
     if (ctx->kernel == LBM_KERNEL_FUSED_COMPACT) return ctx->fplan.ok ? LBM_KERNEL_FUSED_COMPACT : LBM_KERNEL_COMPACT;
     if (ctx->kernel != LBM_KERNEL_AUTO) return ctx->kernel;
-    // small problems: one cooperative launch for the n updates, each thread
+    // instances that fit a thread-block cluster's shared memory stay there for
+    // all n updates, however many instances there are (GB300, FP32, us per
+    // update against two launches each: 16^3 3.1 against 12.3, 16 channels of
+    // 4 x 128 x 4 3.6 against 12.3, 104 slugs of 3840 cells 22.5 against 37.0,
+    // 256 x 16^3 62.7 against 100; in the steady loop's CUDA graphs 4.3 against
+    // 8.6, 4.9 against 9.5, 24.5 against 35.8, 65.9 against 98.4)
+    if (ctx->onchip > 0 && !ctx->slip_on() && n >= 8) return LBM_KERNEL_PERSISTENT;
+    // other small problems: one cooperative launch for the n updates, each thread
     // keeping its cell, beats two launches per update (GB300, FP32, us per
-    // update, stepped from the host: 16^3 5.6 against 12.3, 16 x 16^3 9.3
-    // against 14.4, even at 4 x 32^3; in the steady loop's CUDA graphs, where
-    // launches are cheap: 16^3 6.2 against 7.0, 8 x 16^3 7.3 against 8.0, even
-    // at 16 x 16^3; FP64, stepped: 16^3 28.1 against 34.8, the 16-instance
-    // channel sweep 53.2 against 57.4)
+    // update, stepped from the host: 24^3 5.9 against 12.3, 32^3 6.7 against
+    // 12.3; in the steady loop's CUDA graphs, where launches are cheap: 24^3 7.1
+    // against 8.7, 32^3 8.0 against 9.4; FP64, stepped: 16^3 28.1 against 34.8,
+    // the 16-instance channel sweep 53.2 against 57.4)
     const long long items = (long long)ctx->cfg.batch * ctx->list_max;
     if (ctx->compact_ok && !ctx->slip_on() && n >= 8 &&
         items <= (ctx->in_graph ? kPersistGraphItems : kPersistAutoItems))
@@ -311,6 +318,8 @@ lbm_status plan_fused_compact(lbm_ctx *ctx) {
     return LBM_OK;
 }
 
+StepArgs step_args(lbm_ctx *ctx, int write_macro);
+
 // Lists of the non-solid cells of every instance (in cell order) for the
 // two-pass kernels, and the static pseudo-potential of the SOLID cells, built
 // on the device from the geometry words in ctx->link.  With the compact layout
@@ -354,6 +363,7 @@ lbm_status build_cell_lists(lbm_ctx *ctx) {
     ctx->dfree(rowcnt);
     if (e != cudaSuccess) return ctx->cuda_fail(e, "cell lists");
     ctx->launches += ctx->compact_ok ? 5 : 4;
+    ctx->onchip = ctx->compact_ok ? onchip_threads(step_args(ctx, 0)) : 0;
     return plan_fused_compact(ctx);
 }
 
@@ -407,6 +417,8 @@ StepArgs step_args(lbm_ctx *ctx, int write_macro) {
     a.bar = ctx->bar;
     a.bar_cycles = ctx->bar_cycles;
     a.bar_missing = ctx->bar_missing;
+    // (the failure test of the grid-wide barriers runs the kernel that has them)
+    a.onchip = !a.slip && a.bar_missing == 0 ? ctx->onchip : 0;
     return a;
 }
 
@@ -772,7 +784,7 @@ lbm_status lbm_step(lbm_ctx *ctx, int n) {
             a.ev = ctx->events_for(k);
             cudaError_t e = k == LBM_KERNEL_CLUSTER ? launch_cluster(a, n) : launch_persist(a, n);
             if (e != cudaSuccess) return ctx->cuda_fail(e, "lbm_step persistent launch");
-            if (k == LBM_KERNEL_PERSISTENT) ctx->persist_used = true;
+            if (k == LBM_KERNEL_PERSISTENT && !a.onchip) ctx->persist_used = true;  // (the on-chip kernel has no flag)
             ctx->launches += 1;
             ctx->cur ^= (n & 1);
         }
@@ -1323,7 +1335,7 @@ lbm_status lbm_run_to_steady(lbm_ctx *ctx, int check_every, double tol, int max_
     if (hres) cudaFreeHost(hres);
     cudaStreamDestroy(cs);
     if (e != cudaSuccess) return ctx->cuda_fail(e, "lbm_run_to_steady");
-    if (kres == LBM_KERNEL_PERSISTENT) {
+    if (kres == LBM_KERNEL_PERSISTENT && !step_args(ctx, 0).onchip) {
         ctx->persist_used = true;
         const lbm_status bs = check_barrier(ctx);
         if (bs != LBM_OK) return bs;

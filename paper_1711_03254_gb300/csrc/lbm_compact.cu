@@ -19,6 +19,7 @@
 //   k_collide_c2       S1-S7 for the FP32-arithmetic storages, both components
 //                      as packed FP32 pairs (lbm_pair2.cuh).
 #include "lbm_compact_update.cuh"
+#include "lbm_onchip.cuh"
 
 namespace lbm {
 
@@ -31,6 +32,12 @@ extern template cudaError_t launch_persist_t<double>(const StepArgs &, int);
 extern template cudaError_t launch_persist_t<float>(const StepArgs &, int);
 extern template cudaError_t launch_persist_t<__half>(const StepArgs &, int);
 extern template cudaError_t launch_persist_t<__nv_bfloat16>(const StepArgs &, int);
+extern template int onchip_threads_t<float>(const StepArgs &);
+extern template int onchip_threads_t<__half>(const StepArgs &);
+extern template int onchip_threads_t<__nv_bfloat16>(const StepArgs &);
+extern template cudaError_t launch_onchip_t<float>(const StepArgs &, int);
+extern template cudaError_t launch_onchip_t<__half>(const StepArgs &, int);
+extern template cudaError_t launch_onchip_t<__nv_bfloat16>(const StepArgs &, int);
 
 __global__ void k_compact_links(const uint32_t *__restrict__ list, const int *__restrict__ count,
                                 const uint32_t *__restrict__ link, uint32_t *__restrict__ clink, long long n,
@@ -80,7 +87,24 @@ cudaError_t launch_compact(const StepArgs &a, int parts) {
     return cudaErrorInvalidValue;
 }
 
+int onchip_threads(const StepArgs &a) {
+    switch (a.precision) {
+    case LBM_FP32: return onchip_threads_t<float>(a);
+    case LBM_FP32_F16S: return onchip_threads_t<__half>(a);
+    case LBM_FP32_BF16S: return onchip_threads_t<__nv_bfloat16>(a);
+    default: return 0;
+    }
+}
+
 cudaError_t launch_persist(const StepArgs &a, int nsteps) {
+    if (a.onchip) {
+        switch (a.precision) {
+        case LBM_FP32: return launch_onchip_t<float>(a, nsteps);
+        case LBM_FP32_F16S: return launch_onchip_t<__half>(a, nsteps);
+        case LBM_FP32_BF16S: return launch_onchip_t<__nv_bfloat16>(a, nsteps);
+        default: return cudaErrorInvalidValue;
+        }
+    }
     switch (a.precision) {
     case LBM_FP64: return launch_persist_t<double>(a, nsteps);
     case LBM_FP32: return launch_persist_t<float>(a, nsteps);

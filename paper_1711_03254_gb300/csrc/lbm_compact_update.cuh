@@ -210,6 +210,70 @@ __global__ void __launch_bounds__(kCollideThreads, collide_min_blocks<S>()) k_co
     collide_cell<S, EQ, false>(a, b, k, a.write_macro);
 }
 
+// INLET cell of instance b with geometry word `word` (FP32 arithmetic): the
+// equilibrium at (rho_in, u_in) as deviations from the reference pairs, value i
+// into *at(i).  psi_at(i) is the psi pair of the neighbour in direction i, read
+// only where it is not SOLID.
+template <class S, int EQ, class PsiAt, class At>
+__device__ __forceinline__ void inlet_cell2(const InstParam<float> &p, uint32_t word, PsiAt psi_at, At at) {
+    const float uu = p.u_in[0] * p.u_in[0] + p.u_in[1] * p.u_in[1] + p.u_in[2] * p.u_in[2];
+#pragma unroll
+    for (int i = 0; i < kQ; ++i) {
+        const bool self_ref = i == 0 || ((word >> i) & 1u);
+        const float2 q = self_ref ? make_float2(p.rho_in[0], p.rho_in[1]) : psi_at(i);
+        Pair<S>::store(at(i), feq_dir<float, EQ>(i, p.rho_in[0], p.u_in[0], p.u_in[1], p.u_in[2], uu),
+                       feq_dir<float, EQ>(i, p.rho_in[1], p.u_in[0], p.u_in[1], p.u_in[2], uu),
+                       wgt<float>(i) * ref_value(q.x), wgt<float>(i) * ref_value(q.y));
+    }
+}
+
+// S4-S7 of a cell from its moments: the neighbours' psi pairs (psi_at(i), the
+// cell's own at SOLID neighbours) into the force sums, relaxation, and the
+// stored deviations into *at(i).  psi_own() is read for wall models 0 and 1 only.
+template <class S, int EQ, class PsiAt, class PsiOwn, class At>
+__device__ __forceinline__ Relax<float> relax_cell2(const InstParam<float> &p, int wall_model, uint32_t word,
+                                                    const Moments2 &m, PsiAt psi_at, PsiOwn psi_own_of, At at) {
+    // the stores keep the FP16 reference pair of each direction (the density of
+    // the cell the value streams into; the cell's own at SOLID neighbours)
+    const __half2 rho_h = __float22half2_rn(m.rho);
+    ForceSums2 bs;
+    bs.clear();
+    __half2 Rp[kQ];
+    Rp[0] = rho_h;
+#pragma unroll
+    for (int i = 1; i < kQ; ++i) {
+        const bool solid = (word >> i) & 1u;
+        const float2 q = psi_at(i);
+        bs.add(i, q);
+        Rp[i] = solid ? rho_h : __float22half2_rn(q);
+    }
+    const float2 psi_own = ((word & 0x7FFFEu) && wall_model < 2) ? psi_own_of() : bc2(0.f);
+    const Forces2 F = forces2(bs, psi_own, word, m.rho, p, wall_model);
+    const Relax<float> R = relax2(m, F, p);
+    const Prep2 cp = prep2<EQ>(m, R, F);
+    constexpr float sc = Pair2<S>::kScale;
+    Pair2<S>::store(at(0), rest2<EQ>(cp, __half22float2(Rp[0]), sc));
+#pragma unroll
+    for (int i = 1; i < kQ; i += 2) {
+        float2 vi, vo;
+        pair2<EQ>(cp, i, __half22float2(Rp[i]), __half22float2(Rp[i + 1]), sc, vi, vo);
+        Pair2<S>::store(at(i), vi);
+        Pair2<S>::store(at(i + 1), vo);
+    }
+    return R;
+}
+
+// Fields of the last update (FP32 arithmetic) of the cell with dense index `cell`.
+__device__ __forceinline__ void macro_cell2(const StepArgs &a, int b, long long cell, float r0, float r1, float ux,
+                                            float uy, float uz) {
+    float *mac = (float *)a.macro + (long long)b * 5 * a.g.n;
+    mac[cell] = r0;
+    mac[a.g.n + cell] = r1;
+    mac[2 * a.g.n + cell] = ux;
+    mac[3 * a.g.n + cell] = uy;
+    mac[4 * a.g.n + cell] = uz;
+}
+
 // k_collide_c2: the update of k_collide_c with both components as packed FP32
 // pairs (lbm_pair2.cuh), for the FP32 and 16-bit storages.  Same steps and
 // memory accesses; the neighbour psi pairs enter the force sums unselected
@@ -230,31 +294,16 @@ __device__ __forceinline__ void collide_cell2(const StepArgs &a, int b, uint32_t
     const uint32_t n = a.kmax;
     const float2 *psi = (const float2 *)a.psi + (size_t)b * n;
     __half2 *rout = (__half2 *)a.ref_out + (size_t)b * n;
+    P *fo = (P *)a.f_out + (size_t)b * kQ * n;
+    auto out_at = [&](int i) { return fo + (size_t)i * n + k; };
     const long long cell = c.x + (long long)a.g.nx * (c.y + (long long)a.g.ny * c.z);
-    float *mac = (float *)a.macro + (long long)b * 5 * a.g.n;
     CNbr own_l;
     if constexpr (!PRE) own_l.init(c.x, c.y, c.z, k, instance_tab(a, b), a.words, a.g);
     const CNbr &own = PRE ? *nbr_pre : own_l;
     if (cell_type(word) == kInlet) {
-        // equilibrium at (rho_in, u_in) as deviations from the reference pairs
-        typename Pair<S>::P *fo = (typename Pair<S>::P *)a.f_out + (size_t)b * kQ * n;
-        const float uu = p.u_in[0] * p.u_in[0] + p.u_in[1] * p.u_in[1] + p.u_in[2] * p.u_in[2];
-#pragma unroll
-        for (int i = 0; i < kQ; ++i) {
-            const bool self_ref = i == 0 || ((word >> i) & 1u);
-            const float2 q = self_ref ? make_float2(p.rho_in[0], p.rho_in[1]) : ld_data<COH>(psi + own.dst(i));
-            Pair<S>::store(fo + (size_t)i * n + k, feq_dir<float, EQ>(i, p.rho_in[0], p.u_in[0], p.u_in[1], p.u_in[2], uu),
-                           feq_dir<float, EQ>(i, p.rho_in[1], p.u_in[0], p.u_in[1], p.u_in[2], uu),
-                           wgt<float>(i) * ref_value(q.x), wgt<float>(i) * ref_value(q.y));
-        }
+        inlet_cell2<S, EQ>(p, word, [&](int i) { return ld_data<COH>(psi + own.dst(i)); }, out_at);
         rout[k] = __floats2half2_rn(p.rho_in[0], p.rho_in[1]);
-        if (write_macro) {
-            mac[cell] = p.rho_in[0];
-            mac[a.g.n + cell] = p.rho_in[1];
-            mac[2 * a.g.n + cell] = p.u_in[0];
-            mac[3 * a.g.n + cell] = p.u_in[1];
-            mac[4 * a.g.n + cell] = p.u_in[2];
-        }
+        if (write_macro) macro_cell2(a, b, cell, p.rho_in[0], p.rho_in[1], p.u_in[0], p.u_in[1], p.u_in[2]);
         return;
     }
     // the psi pairs of the 18 neighbours (the cell's own at SOLID ones) start
@@ -272,7 +321,6 @@ __device__ __forceinline__ void collide_cell2(const StepArgs &a, int b, uint32_t
     }
     if constexpr (!COH) cp_async_commit_group();
     const P *f = (const P *)a.f_in + (size_t)b * kQ * n;
-    P *fo = (P *)a.f_out + (size_t)b * kQ * n;
     Moments2 m;
     auto pull = [&](const CNbr &nb, uint32_t sk, uint32_t sw) {
         float2 v[kQ];
@@ -292,43 +340,11 @@ __device__ __forceinline__ void collide_cell2(const StepArgs &a, int b, uint32_t
             pull(own, k, word);
         }
     }
-    // psi pairs of the 18 neighbours into the force sums; the stores keep the
-    // FP16 reference pair of each direction (the density of the cell the
-    // value streams into; the cell's own at SOLID neighbours)
-    const __half2 rho_h = __float22half2_rn(m.rho);
-    ForceSums2 bs;
-    bs.clear();
-    __half2 Rp[kQ];
-    Rp[0] = rho_h;
     if constexpr (!COH) cp_async_wait_all();
-#pragma unroll
-    for (int i = 1; i < kQ; ++i) {
-        const bool solid = (word >> i) & 1u;
-        const float2 q = qs[i - 1][tid];
-        bs.add(i, q);
-        Rp[i] = solid ? rho_h : __float22half2_rn(q);
-    }
-    const float2 psi_own = ((word & 0x7FFFEu) && a.wall_model < 2) ? ld_data<COH>(psi + k) : bc2(0.f);
-    const Forces2 F = forces2(bs, psi_own, word, m.rho, p, a.wall_model);
-    const Relax<float> R = relax2(m, F, p);
-    const Prep2 cp = prep2<EQ>(m, R, F);
-    constexpr float sc = Pair2<S>::kScale;
-    Pair2<S>::store(fo + k, rest2<EQ>(cp, __half22float2(Rp[0]), sc));
-#pragma unroll
-    for (int i = 1; i < kQ; i += 2) {
-        float2 vi, vo;
-        pair2<EQ>(cp, i, __half22float2(Rp[i]), __half22float2(Rp[i + 1]), sc, vi, vo);
-        Pair2<S>::store(fo + (size_t)i * n + k, vi);
-        Pair2<S>::store(fo + (size_t)(i + 1) * n + k, vo);
-    }
-    rout[k] = rho_h;
-    if (write_macro) {
-        mac[cell] = m.rho.x;
-        mac[a.g.n + cell] = m.rho.y;
-        mac[2 * a.g.n + cell] = R.ux;
-        mac[3 * a.g.n + cell] = R.uy;
-        mac[4 * a.g.n + cell] = R.uz;
-    }
+    const Relax<float> R = relax_cell2<S, EQ>(p, a.wall_model, word, m, [&](int i) { return qs[i - 1][tid]; },
+                                              [&]() { return ld_data<COH>(psi + k); }, out_at);
+    rout[k] = __float22half2_rn(m.rho);
+    if (write_macro) macro_cell2(a, b, cell, m.rho.x, m.rho.y, R.ux, R.uy, R.uz);
 }
 
 template <class S, int EQ>

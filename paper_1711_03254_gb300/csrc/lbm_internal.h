@@ -19,6 +19,7 @@ struct StepArgs {
     unsigned *bar = nullptr;  // persistent update: barrier counter and give-up flag (2 words)
     long long bar_cycles = 0; // its barriers' bound on a wait, in SM clock cycles
     unsigned bar_missing = 0; // arrivals its barriers wait for beyond the grid (failure test: > 0)
+    int onchip = 0;           // persistent update: threads per block of the on-chip kernel (0: not that one)
     int batch;
     Grid g;
     const void *f_in;
@@ -104,6 +105,8 @@ int fused_tile_count();
 // nsteps updates in one persistent launch, one thread-block cluster per instance
 cudaError_t launch_cluster(const StepArgs &a, int nsteps);
 cudaError_t launch_persist(const StepArgs &a, int nsteps);
+// threads per block of the on-chip persistent update (lbm_onchip.cuh); 0 where it does not apply
+int onchip_threads(const StepArgs &a);
 int cluster_size_for(long long n);
 cudaError_t launch_init(const InitArgs &a);
 cudaError_t launch_links(const uint8_t *type, uint32_t *link, const Grid &g, int batch, cudaStream_t s);

@@ -164,3 +164,45 @@ def test_batched_small_instances_timing(lbm):
             sim.close()
         rows.append((shape, B, prec, ms))
     print("ms per update:", rows)
+
+
+ONCHIP = [
+    # nx, ny, nz, instances: cells around the blocks' sizes (64 .. 512 threads, up to 16 blocks)
+    (1, 1, 1, 1), (7, 9, 1, 3), (8, 8, 1, 2), (13, 5, 1, 1), (16, 16, 4, 2), (5, 41, 5, 1), (16, 16, 16, 1),
+    (17, 16, 15, 40), (128, 32, 1, 30), (20, 20, 20, 2), (31, 24, 11, 3), (32, 16, 16, 1),
+]
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp16s", "bf16s"])
+@pytest.mark.parametrize("dims", ONCHIP, ids=lambda d: "x".join(map(str, d)))
+def test_onchip_update_equals_two_launches(lbm, dims, prec):
+    """Instances of at most 8192 cells stay in shared memory for all n updates:
+    the state after odd and even n equals the two-launch update's, bit for bit,
+    over all block sizes, batches of one and of several waves of clusters,
+    INLET / OUTLET planes and instances with different geometries."""
+    nx, ny, nz, B = dims
+    rng = np.random.default_rng(sum(dims))
+    shape = (B, nz, ny, nx)
+    t = (rng.random(shape) < 0.2).astype(np.uint8)
+    t[:, 0, 0, 0] = 0
+    if nx > 30:
+        t[..., 0][t[..., 0] != 1] = 2
+        t[..., -1][t[..., -1] != 1] = 3
+    r1, r2 = 0.4 + 0.3 * rng.random(shape), 0.4 + 0.3 * rng.random(shape)
+    u = 0.02 * (rng.random(shape + (3,)) - 0.5)
+    solid = t == 1
+    r1[solid] = r2[solid] = 0.0
+    u[solid] = 0.0
+    params = [dict(tau=(0.8, 1.0 + 0.02 * b), G=-0.7, rho_s=0.1 * (b % 3 - 1), g=(1e-6, 2e-6, -1e-6),
+                   rho_in=(0.6, 0.4), u_in=(0.01, 0.0, 0.0)) for b in range(B)]
+    out = []
+    for kernel in ("persistent", "compact"):
+        sim = lbm.Sim(nx, ny, nz, params, precision=prec, kernel=kernel, eq_order=nz % 2, reg_order=2 + ny % 2)
+        sim.set_geometry(t)
+        sim.set_fields(r1, r2, u)
+        sim.step(3)
+        sim.step(4)
+        out.append((sim.get_f(),) + sim.get_fields())
+        sim.close()
+    for a, b in zip(*out):
+        np.testing.assert_array_equal(a, b)
