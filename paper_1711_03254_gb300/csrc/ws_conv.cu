@@ -78,6 +78,18 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t saddr, uint32_t lbo, uint
     return d;                // base offset 0, layout type 0 (no swizzle)
 }
 
+// shared-memory matrix descriptor: 32-byte swizzle (layout type 6), K-major rows
+// of 32 bytes, 8-row groups 256 B apart
+__device__ __forceinline__ uint64_t umma_desc_sw32(uint32_t saddr) {
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
+    d |= (uint64_t)1 << 16;
+    d |= (uint64_t)(256u >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)6 << 61;
+    return d;
+}
+
 // instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, both K-major
 __host__ __device__ constexpr uint32_t umma_idesc_bf16(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
@@ -365,11 +377,7 @@ __global__ void __launch_bounds__(RTHREADS) k_conv3_fwd_res(const __grid_constan
                          : "memory");
             const uint32_t sa = base + (uint32_t)st * pl.stage_bytes, sb = sa + 2 * pl.a_half;
             tma_load_5d(sa, &xmap, c * 16, -1, y0 - 1, z + dz - 1, n, fb);
-            tma_load_5d(sa + pl.a_half, &xmap, c * 16 + 8, -1, y0 - 1, z + dz - 1, n, fb);
-            for (int t9 = 0; t9 < 9; ++t9)
-                for (int h = 0; h < 2; ++h)
-                    tma_load_3d(sb + (uint32_t)(t9 * 2 + h) * (uint32_t)Co * 16u, &wmap, c * 16 + 8 * h, dz * 9 + t9,
-                                0, fb);
+            tma_load_3d(sb, &wmap, c * 16, 0, dz * 9, fb);
             issued = s + 1;
         }
         // wait for the loads still in flight (the last phase issued on each stage)
@@ -390,15 +398,15 @@ __global__ void __launch_bounds__(RTHREADS) k_conv3_fwd_res(const __grid_constan
             const uint32_t sa = base + (uint32_t)st * pl.stage_bytes, sb = sa + 2 * pl.a_half;
             // descriptors of the taps: a base descriptor's start-address field (16-byte
             // units) plus the tap's offset (all addresses stay below 256 KB)
-            const uint64_t ad0 = umma_desc(sa, pl.a_half, 128), bd0 = umma_desc(sb, (uint32_t)Co * 16u, 128);
+            const uint64_t ad0 = umma_desc_sw32(sa), bd0 = umma_desc_sw32(sb);
             const uint32_t pitch = (uint32_t)pl.pitch, bstep = 2u * (uint32_t)Co;
             for (int j = 0; j < nt; ++j) {
-                const uint64_t aj = ad0 + (uint64_t)(128 * j);
+                const uint64_t aj = ad0 + (uint64_t)(256 * j);
                 const uint32_t dj = tmem + (uint32_t)(j * Co);
 #pragma unroll
                 for (int t9 = 0; t9 < 9; ++t9) {
                     const uint32_t dy = (uint32_t)(t9 / 3), dx = (uint32_t)(t9 % 3);
-                    const uint64_t ad = aj + (uint64_t)(dy * pitch + dx);
+                    const uint64_t ad = aj + (uint64_t)(2u * (dy * pitch + dx));
                     const uint64_t bd = bd0 + (uint64_t)((uint32_t)t9 * bstep);
                     const uint32_t acc = (s > 0 || t9 > 0) ? 1u : 0u;
                     asm volatile(
@@ -572,11 +580,7 @@ __global__ void __launch_bounds__(PTHREADS, 1) k_conv3_fwd_pers(const __grid_con
                              : "memory");
                 const uint32_t sa = base + (uint32_t)st * pl.stage_bytes, sb = sa + 2 * pl.a_half;
                 tma_load_5d(sa, &xmap, c * 16, -1, r.y0 - 1, r.z + dz - 1, r.n, fb);
-                tma_load_5d(sa + pl.a_half, &xmap, c * 16 + 8, -1, r.y0 - 1, r.z + dz - 1, r.n, fb);
-                for (int t9 = 0; t9 < 9; ++t9)
-                    for (int h = 0; h < 2; ++h)
-                        tma_load_3d(sb + (uint32_t)(t9 * 2 + h) * (uint32_t)Co * 16u, &wmap, c * 16 + 8 * h,
-                                    dz * 9 + t9, 0, fb);
+                tma_load_3d(sb, &wmap, c * 16, 0, dz * 9, fb);
                 issued = g + 1;
             }
         }
@@ -610,15 +614,15 @@ __global__ void __launch_bounds__(PTHREADS, 1) k_conv3_fwd_pers(const __grid_con
                 const uint32_t sa = base + (uint32_t)st * pl.stage_bytes, sb = sa + 2 * pl.a_half;
                 // descriptors of the taps: the start-address field (16-byte units) of a base
                 // descriptor plus the tap's offset (all addresses stay below 256 KB)
-                const uint64_t ad0 = umma_desc(sa, pl.a_half, 128), bd0 = umma_desc(sb, (uint32_t)Co * 16u, 128);
+                const uint64_t ad0 = umma_desc_sw32(sa), bd0 = umma_desc_sw32(sb);
                 const uint32_t pitch = (uint32_t)pl.pitch, bstep = 2u * (uint32_t)Co;
                 for (int j = 0; j < r.nt; ++j) {
-                    const uint64_t aj = ad0 + (uint64_t)(128 * j);
+                    const uint64_t aj = ad0 + (uint64_t)(256 * j);
                     const uint32_t dj = dbase + (uint32_t)(j * Co);
 #pragma unroll
                     for (int t9 = 0; t9 < 9; ++t9) {
                         const uint32_t dy = (uint32_t)(t9 / 3), dx = (uint32_t)(t9 % 3);
-                        const uint64_t ad = aj + (uint64_t)(dy * pitch + dx);
+                        const uint64_t ad = aj + (uint64_t)(2u * (dy * pitch + dx));
                         const uint64_t bd = bd0 + (uint64_t)((uint32_t)t9 * bstep);
                         const uint32_t acc = (s > 0 || t9 > 0) ? 1u : 0u;
                         asm volatile(
@@ -1488,16 +1492,17 @@ static size_t res_smem_request(const ResPlan &p) {
     return s;
 }
 
-static bool act_map(CUtensorMap *map, const void *t, int ld, const Act &a, int C, int box_x, int box_y) {
+static bool act_map(CUtensorMap *map, const void *t, int ld, const Act &a, int C, int box_c, int box_x, int box_y,
+                    CUtensorMapSwizzle swizzle) {
     EncodeTiledFn enc = encode_tiled();
     if (!enc) return false;
     const cuuint64_t dim[5] = {(cuuint64_t)C, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)a.D, (cuuint64_t)a.N};
     const cuuint64_t row = (cuuint64_t)ld * 2;
     const cuuint64_t str[4] = {row, row * a.W, row * a.W * a.H, row * a.W * a.H * a.D};
-    const cuuint32_t box[5] = {8, (cuuint32_t)box_x, (cuuint32_t)box_y, 1, 1};
+    const cuuint32_t box[5] = {(cuuint32_t)box_c, (cuuint32_t)box_x, (cuuint32_t)box_y, 1, 1};
     const cuuint32_t ones[5] = {1, 1, 1, 1, 1};
     return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void *>(t), dim, str, box, ones,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -1532,13 +1537,14 @@ static int conv3_fwd_res(const void *x, int ldx, const void *w, const float *bia
                          const Act &a, int Ci, int Co, int relu, cudaStream_t s, const ResPlan &pl) {
     EncodeTiledFn enc = encode_tiled();
     CUtensorMap xmap, wmap;
-    if (!enc || !act_map(&xmap, x, ldx, a, Ci, pl.pitch, pl.by + 2)) return 2;
+    if (!enc || !act_map(&xmap, x, ldx, a, Ci, 16, pl.pitch, pl.by + 2, CU_TENSOR_MAP_SWIZZLE_32B)) return 2;
+    // the weights as [tap][Co][Ci], 16 channels of all Co for nine taps at a time
     const cuuint32_t ones[3] = {1, 1, 1};
-    const cuuint64_t wdim[3] = {(cuuint64_t)Ci, 27, (cuuint64_t)Co};
-    const cuuint64_t wstr[2] = {(cuuint64_t)Ci * 2, (cuuint64_t)Ci * 2 * 27};
-    const cuuint32_t wbox[3] = {8, 1, (cuuint32_t)Co};
+    const cuuint64_t wdim[3] = {(cuuint64_t)Ci, (cuuint64_t)Co, 27};
+    const cuuint64_t wstr[2] = {(cuuint64_t)Ci * 2 * 27, (cuuint64_t)Ci * 2};
+    const cuuint32_t wbox[3] = {16, (cuuint32_t)Co, 9};
     if (enc(&wmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(w), wdim, wstr, wbox, ones,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return 2;
     const size_t smem = res_smem_request(pl);
@@ -1714,8 +1720,8 @@ static size_t wg_smem_request(const WgPlan &p) {
 static int conv3_wgrad_res(const void *x, int ldx, const void *dy, int ldy, float *part, float *bpart, const Act &a,
                            int Ci, int Co, cudaStream_t s, const WgPlan &pl, bool dz_slots) {
     CUtensorMap xmap, dymap;
-    if (!act_map(&xmap, x, ldx, a, Ci, pl.pitch, dz_slots ? pl.by + 2 : pl.by) ||
-        !act_map(&dymap, dy, ldy, a, Co, pl.pitch, pl.by))
+    if (!act_map(&xmap, x, ldx, a, Ci, 8, pl.pitch, dz_slots ? pl.by + 2 : pl.by, CU_TENSOR_MAP_SWIZZLE_NONE) ||
+        !act_map(&dymap, dy, ldy, a, Co, 8, pl.pitch, pl.by, CU_TENSOR_MAP_SWIZZLE_NONE))
         return 2;
     const size_t smem = wg_smem_request(pl);
     static size_t attr[2] = {0, 0};
