@@ -90,6 +90,18 @@ __device__ __forceinline__ uint64_t umma_desc_sw32(uint32_t saddr) {
     return d;
 }
 
+// the same swizzle for an MN-major operand: 32-byte rows of 16 channels per
+// position, 8 positions 256 B apart, 16-channel groups `group` bytes apart
+__device__ __forceinline__ uint64_t umma_desc_mn32(uint32_t saddr, uint32_t group) {
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
+    d |= (uint64_t)((group >> 4) & 0x3FFFu) << 16;
+    d |= (uint64_t)(256u >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)6 << 61;
+    return d;
+}
+
 // instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, both K-major
 __host__ __device__ constexpr uint32_t umma_idesc_bf16(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
@@ -931,7 +943,7 @@ __global__ void __launch_bounds__(RTHREADS) k_conv3_wgrad_res(const __grid_const
     extern __shared__ __align__(128) unsigned char sm_raw[];
     unsigned char *sm = sm_raw + ((1024u - (smem_u32(sm_raw) & 1023u)) & 1023u);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int NS = pl.stages, G = pl.ci_blk / 8, NB = Co / 8;
+    const int NS = pl.stages, G = pl.ci_blk / 16, NB = Co / 16;
     uint64_t *full = reinterpret_cast<uint64_t *>(sm + (size_t)NS * pl.stage_bytes);
     uint64_t *empty = full + NS;
     uint64_t *done = empty + NS;
@@ -943,7 +955,8 @@ __global__ void __launch_bounds__(RTHREADS) k_conv3_wgrad_res(const __grid_const
     const int kb0 = pb * pl.kpb, kb1 = min(kb0 + pl.kpb, nkb);
     const int nsteps = kb1 > kb0 ? kb1 - kb0 : 0;
     const int nreal = min(pl.J, 9 - ti * pl.J);  // tap pairs of this tile (>= 1)
-    const uint32_t tx = (uint32_t)(nreal * G + NB) * (uint32_t)(pl.by * pl.pitch) * 16u;
+    const uint32_t tx = (uint32_t)(nreal * G + NB) * (uint32_t)(pl.by * pl.pitch) * 32u;
+    const uint32_t group = 2 * pl.region;  // bytes of a 16-channel group
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tslot)),
@@ -961,10 +974,10 @@ __global__ void __launch_bounds__(RTHREADS) k_conv3_wgrad_res(const __grid_const
     const int jb = (bpart && cb == 0 && ti == pl.ntile - 1 && nreal < pl.J) ? nreal : -1;
     {
         uint4 *z4 = reinterpret_cast<uint4 *>(sm);
-        const uint32_t n16 = (uint32_t)NS * pl.stage_bytes / 16u, per_region = pl.region / 16u;
+        const uint32_t n16 = (uint32_t)NS * pl.stage_bytes / 16u, per_group = group / 16u;
         const uint32_t per_stage = pl.stage_bytes / 16u, ones = 0x3F803F80u;  // BF16 1.0 twice
         for (uint32_t i = tid; i < n16; i += RTHREADS) {
-            const bool one = jb >= 0 && (i % per_stage) / per_region == (uint32_t)(jb * G);
+            const bool one = jb >= 0 && (i % per_stage) / per_group == (uint32_t)(jb * G);
             z4[i] = one ? make_uint4(ones, ones, ones, ones) : make_uint4(0u, 0u, 0u, 0u);
         }
     }
@@ -993,11 +1006,11 @@ __global__ void __launch_bounds__(RTHREADS) k_conv3_wgrad_res(const __grid_const
             for (int j = 0; j < nreal; ++j) {
                 const int m = ti * pl.J + j, dz = m / 3, dy = m - 3 * dz;
                 for (int g = 0; g < G; ++g)
-                    tma_load_5d(sa + (uint32_t)(j * G + g) * pl.region, &xmap, cb * pl.ci_blk + 8 * g, -1,
+                    tma_load_5d(sa + (uint32_t)(j * G + g) * group, &xmap, cb * pl.ci_blk + 16 * g, -1,
                                 y0 + dy - 1, z + dz - 1, n, fb);
             }
             for (int g = 0; g < NB; ++g)
-                tma_load_5d(sa + (uint32_t)(16 + g) * pl.region, &dymap, 8 * g, 0, y0, z, n, fb);
+                tma_load_5d(sa + (uint32_t)(8 + g) * group, &dymap, 16 * g, 0, y0, z, n, fb);
             issued = s + 1;
         }
         for (int st = 0; st < NS && st < issued; ++st) {
@@ -1014,11 +1027,11 @@ __global__ void __launch_bounds__(RTHREADS) k_conv3_wgrad_res(const __grid_const
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
-            const uint32_t sa = base + (uint32_t)st * pl.stage_bytes, sb = sa + 16u * pl.region;
+            const uint32_t sa = base + (uint32_t)st * pl.stage_bytes, sb = sa + 8u * group;
             for (int ks = 0; ks < pl.ksteps; ++ks) {
-                const uint64_t bd = umma_desc(sb + (uint32_t)ks * 256u, 128, pl.region);
+                const uint64_t bd = umma_desc_mn32(sb + (uint32_t)ks * 512u, group);
                 for (int dx = 0; dx < 3; ++dx) {
-                    const uint64_t ad = umma_desc(sa + (uint32_t)(ks * 16 + dx) * 16u, 128, pl.region);
+                    const uint64_t ad = umma_desc_mn32(sa + (uint32_t)(ks * 16 + dx) * 32u, group);
                     const uint32_t acc = (s > 0 || ks > 0) ? 1u : 0u;
                     asm volatile(
                         "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
@@ -1720,8 +1733,10 @@ static size_t wg_smem_request(const WgPlan &p) {
 static int conv3_wgrad_res(const void *x, int ldx, const void *dy, int ldy, float *part, float *bpart, const Act &a,
                            int Ci, int Co, cudaStream_t s, const WgPlan &pl, bool dz_slots) {
     CUtensorMap xmap, dymap;
-    if (!act_map(&xmap, x, ldx, a, Ci, 8, pl.pitch, dz_slots ? pl.by + 2 : pl.by, CU_TENSOR_MAP_SWIZZLE_NONE) ||
-        !act_map(&dymap, dy, ldy, a, Co, 8, pl.pitch, pl.by, CU_TENSOR_MAP_SWIZZLE_NONE))
+    const int box_c = dz_slots ? 8 : 16;
+    const CUtensorMapSwizzle swz = dz_slots ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_32B;
+    if (!act_map(&xmap, x, ldx, a, Ci, box_c, pl.pitch, dz_slots ? pl.by + 2 : pl.by, swz) ||
+        !act_map(&dymap, dy, ldy, a, Co, box_c, pl.pitch, pl.by, swz))
         return 2;
     const size_t smem = wg_smem_request(pl);
     static size_t attr[2] = {0, 0};
