@@ -70,7 +70,8 @@ int ws_conv3d_flip_weights(const void *w, void *wf, int Co, int Ci, int k, void 
  *    whole lines, M = 128 rows of (tap pair (dz, dy), channel) loaded by TMA
  *    as line boxes, the three dx taps as shifted views of the same boxes; for
  *    Ci a multiple of 32 and Co <= 48, M = (dz, channel) rows of boxes with
- *    halo lines instead, and all nine (dy, dx) taps are shifted views;
+ *    halo lines instead, the dy taps shifted views of them and the dx taps
+ *    three copies of dy side by side (N = 3 Co);
  *  - gathered rows (k = 1, and k = 3 where no resident plan fits): rows
  *    (tap, ci) in tiles of 128, K = chunks of 4096 positions gathered with
  *    16-byte copies.
@@ -87,7 +88,8 @@ int ws_conv3d_bwd_weight(const void *x, int ldx, const void *dy, int ldy, float 
 /* Selects the weight-gradient kernel of later ws_conv3d_bwd_weight calls
  * (process-wide): 0 automatic (resident tiles where a plan fits, else
  * gathered rows), 1 gathered rows always, 2 resident tiles always for k = 3
- * (a call that no plan fits then returns 1), 3 as 2 but with tap-pair rows
+ * (a call that no plan fits then returns 1) and no copies of dy (all nine
+ * (dy, dx) taps as shifted views), 3 as 2 but with tap-pair rows
  * only (never the (dz, channel) rows).  Returns the previous choice, or -1
  * for an unknown value (nothing changes). */
 int ws_conv3d_bwd_weight_algo(int algo);
@@ -100,7 +102,8 @@ int ws_conv3d_bwd_weight_algo(int algo);
  * columns, blocks per SM, bytes of one K half of a stage's input, stage bytes,
  * TMA bytes per stage, dynamic shared memory requested, blocks in the grid,
  * columns per accumulator buffer (persistent kernel, else 0).  which = 1:
- * weight gradient; out[0..15] = dz-slot kernel (0/1), lines per K-block,
+ * weight gradient; out[0..15] = dz-slot kernel (0: none, 1: without, 2: with
+ * copies of dy), lines per K-block,
  * K-blocks per plane, line pitch, K-steps per K-block, tap slots per M tile,
  * channels per M group, M tiles per channel block, position blocks, K-blocks
  * per position block, stages, tensor-memory columns, region bytes, stage

@@ -1109,6 +1109,17 @@ __global__ void __launch_bounds__(RTHREADS) k_conv3_wgrad_res(const __grid_const
 // then the dY regions, padded with zero regions up to 16; all regions have
 // the same size, so the 16 M groups are one stride byte offset apart.
 // Partials, bounded waits and roles as in k_conv3_wgrad_res.
+//
+// COPIES (the automatic choice): the dx taps come from three copies of dY,
+// loaded 0, 1 and 2 columns to the left, side by side as N = (dx, Co), so a K-step
+// is three MMAs of N = 3 Co, one per dy (A rows shifted by dy (W + 2)), instead of
+// nine of N = Co.  At N = 32 an MMA costs about 80 clocks, most of it reading
+// the 4 KB of A; at N = 96 three times the work reads A once.  (dY[q - dx] is zero
+// in the padding columns, so the row order (line, column) keeps every product of
+// the sum.)  Tiles have 32-byte rows of 16 channels in the 32-byte swizzle; per
+// stage 6 X groups, the ones, then the dY groups (copy, Co / 16).  64^3 32->32:
+// 109 us against 181 without the copies, 96->32 252 against 460.
+template <bool COPIES>
 __global__ void __launch_bounds__(RTHREADS) k_conv3_wgrad_dz(const __grid_constant__ CUtensorMap xmap,
                                                             const __grid_constant__ CUtensorMap dymap,
                                                             float *__restrict__ part, float *__restrict__ bpart,
@@ -1116,7 +1127,7 @@ __global__ void __launch_bounds__(RTHREADS) k_conv3_wgrad_dz(const __grid_consta
     extern __shared__ __align__(128) unsigned char sm_raw[];
     unsigned char *sm = sm_raw + ((1024u - (smem_u32(sm_raw) & 1023u)) & 1023u);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int NS = pl.stages, NB = Co / 8;
+    const int NS = pl.stages, NB = Co / (COPIES ? 16 : 8);
     uint64_t *full = reinterpret_cast<uint64_t *>(sm + (size_t)NS * pl.stage_bytes);
     uint64_t *empty = full + NS;
     uint64_t *done = empty + NS;
@@ -1128,7 +1139,10 @@ __global__ void __launch_bounds__(RTHREADS) k_conv3_wgrad_dz(const __grid_consta
     const int kb0 = pb * pl.kpb, kb1 = min(kb0 + pl.kpb, nkb);
     const int nsteps = kb1 > kb0 ? kb1 - kb0 : 0;
     const uint32_t rows_x = (uint32_t)((pl.by + 2) * pl.pitch), rows_y = (uint32_t)(pl.by * pl.pitch);
-    const uint32_t tx = (12u * rows_x + (uint32_t)NB * rows_y) * 16u;
+    const uint32_t tx = COPIES ? (6u * rows_x + 3u * (uint32_t)NB * rows_y) * 32u
+                               : (12u * rows_x + (uint32_t)NB * rows_y) * 16u;
+    // COPIES: bytes of a 16-channel group of X and of dY (or of the ones); dY's offset in a stage
+    const uint32_t gx = 2 * pl.region, gy = (uint32_t)pl.ksteps * 512u, y_off = 6 * gx + gy;
     const bool fold = bpart && cb == 0;
 
     if (warp == 0) {
@@ -1148,7 +1162,9 @@ __global__ void __launch_bounds__(RTHREADS) k_conv3_wgrad_dz(const __grid_consta
         const uint32_t n16 = (uint32_t)NS * pl.stage_bytes / 16u, per_region = pl.region / 16u;
         const uint32_t per_stage = pl.stage_bytes / 16u, ones = 0x3F803F80u;  // BF16 1.0 twice
         for (uint32_t i = tid; i < n16; i += RTHREADS) {
-            const bool one = fold && (i % per_stage) / per_region == 12u;
+            const uint32_t at = i % per_stage;
+            const bool one =
+                fold && (COPIES ? at >= 6 * gx / 16u && at < y_off / 16u : at / per_region == 12u);
             z4[i] = one ? make_uint4(ones, ones, ones, ones) : make_uint4(0u, 0u, 0u, 0u);
         }
     }
@@ -1173,12 +1189,22 @@ __global__ void __launch_bounds__(RTHREADS) k_conv3_wgrad_dz(const __grid_consta
             const uint32_t fb = smem_u32(&full[st]);
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(fb), "r"(tx) : "memory");
             const uint32_t sa = base + (uint32_t)st * pl.stage_bytes;
-            for (int dz = 0; dz < 3; ++dz)
-                for (int g = 0; g < 4; ++g)
-                    tma_load_5d(sa + (uint32_t)(dz * 4 + g) * pl.region, &xmap, cb * 32 + 8 * g, -1, y0 - 1,
-                                z + dz - 1, n, fb);
-            for (int g = 0; g < NB; ++g)
-                tma_load_5d(sa + (uint32_t)(13 + g) * pl.region, &dymap, 8 * g, 0, y0, z, n, fb);
+            if constexpr (COPIES) {
+                for (int dz = 0; dz < 3; ++dz)
+                    for (int g = 0; g < 2; ++g)
+                        tma_load_5d(sa + (uint32_t)(dz * 2 + g) * gx, &xmap, cb * 32 + 16 * g, -1, y0 - 1, z + dz - 1,
+                                    n, fb);
+                for (int dx = 0; dx < 3; ++dx)
+                    for (int g = 0; g < NB; ++g)
+                        tma_load_5d(sa + y_off + (uint32_t)(dx * NB + g) * gy, &dymap, 16 * g, -dx, y0, z, n, fb);
+            } else {
+                for (int dz = 0; dz < 3; ++dz)
+                    for (int g = 0; g < 4; ++g)
+                        tma_load_5d(sa + (uint32_t)(dz * 4 + g) * pl.region, &xmap, cb * 32 + 8 * g, -1, y0 - 1,
+                                    z + dz - 1, n, fb);
+                for (int g = 0; g < NB; ++g)
+                    tma_load_5d(sa + (uint32_t)(13 + g) * pl.region, &dymap, 8 * g, 0, y0, z, n, fb);
+            }
             issued = s + 1;
         }
         for (int st = 0; st < NS && st < issued; ++st) {
@@ -1187,7 +1213,7 @@ __global__ void __launch_bounds__(RTHREADS) k_conv3_wgrad_dz(const __grid_consta
         }
     } else if (tid == 32) {
         // MN-major A and B (bits 15, 16), FP32 accumulator, BF16 operands
-        const uint32_t idesc = umma_idesc_bf16(128, Co) | (1u << 15) | (1u << 16);
+        const uint32_t idesc = umma_idesc_bf16(128, COPIES ? 3 * Co : Co) | (1u << 15) | (1u << 16);
         for (int s = 0; s < nsteps; ++s) {
             const int st = s % NS;
             if (!mbar_wait(smem_u32(&full[st]), (uint32_t)((s / NS) & 1))) {
@@ -1195,13 +1221,15 @@ __global__ void __launch_bounds__(RTHREADS) k_conv3_wgrad_dz(const __grid_consta
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
-            const uint32_t sa = base + (uint32_t)st * pl.stage_bytes, sb = sa + 13u * pl.region;
+            const uint32_t sa = base + (uint32_t)st * pl.stage_bytes, sb = sa + (COPIES ? y_off : 13u * pl.region);
             for (int ks = 0; ks < pl.ksteps; ++ks) {
-                const uint64_t bd = umma_desc(sb + (uint32_t)ks * 256u, 128, pl.region);
-                for (int t9 = 0; t9 < 9; ++t9) {
+                const uint64_t bd = COPIES ? umma_desc_mn32(sb + (uint32_t)ks * 512u, gy)
+                                           : umma_desc(sb + (uint32_t)ks * 256u, 128, pl.region);
+                for (int t9 = 0; t9 < 9; t9 += COPIES ? 3 : 1) {
                     const int dy = t9 / 3, dx = t9 - 3 * dy;
                     const uint64_t ad =
-                        umma_desc(sa + (uint32_t)(ks * 16 + dy * pl.pitch + dx) * 16u, 128, pl.region);
+                        COPIES ? umma_desc_mn32(sa + (uint32_t)(ks * 16 + dy * pl.pitch) * 32u, gx)
+                               : umma_desc(sa + (uint32_t)(ks * 16 + dy * pl.pitch + dx) * 16u, 128, pl.region);
                     const uint32_t acc = (s > 0 || ks > 0) ? 1u : 0u;
                     asm volatile(
                         "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
@@ -1603,7 +1631,8 @@ static int conv3_fwd_res(const void *x, int ldx, const void *w, const float *bia
     return cudaGetLastError() == cudaSuccess ? 0 : 2;
 }
 
-// weight-gradient kernel choice: 0 automatic, 1 gathered rows (k_conv_wgrad_tc), 2 resident tiles
+// weight-gradient kernel choice: 0 automatic (k_conv3_wgrad_dz with copies of dY where it applies, else
+// k_conv3_wgrad_res), 1 gathered rows (k_conv_wgrad_tc), 2 resident tiles with the dz slots but no copies
 // (k_conv3_wgrad_dz where it applies, else k_conv3_wgrad_res), 3 resident tiles without the dz slots
 // (k_conv3_wgrad_res only)
 static int g_wgrad_algo = 0;
@@ -1720,6 +1749,63 @@ static bool wg_dz_plan(const Act &a, int Ci, int Co, WgPlan &p) {
     return by_blocks <= 65535;
 }
 
+// Plan of k_conv3_wgrad_dz with three copies of dY (same conditions): as
+// wg_dz_plan, with X groups of (by + 2) lines and the rows the dy shift of the
+// last K-step reaches, dY groups of whole K-steps, and stages that also cover
+// what the eighth M group (dropped rows) reads.  `region` is half an X group.
+static bool wg_copies_plan(const Act &a, int Ci, int Co, WgPlan &p) {
+    const int pitch = a.W + 2;
+    if (pitch > 256 || Ci % 32 || Co > 48) return false;
+    p.ci_blk = 32;
+    p.J = 4;
+    p.ntile = 1;
+    p.pitch = pitch;
+    p.cols = 32;
+    while (p.cols < 9 * Co) p.cols *= 2;
+    bool found = false;
+    int resident = 1;
+    for (int by = std::max(1, std::min(a.H, 132 / pitch)); by >= 1 && !found; --by) {
+        if (by + 2 > 256) continue;
+        p.by = by;
+        p.ksteps = (by * pitch + 15) / 16;
+        const int rb = (std::max((by + 2) * pitch, p.ksteps * 16 + 2 * pitch) + 7) / 8 * 8;
+        p.region = (uint32_t)rb * 16u;
+        const uint32_t gy = (uint32_t)p.ksteps * 512u;
+        p.stage_bytes = std::max(12 * p.region + (1 + 3 * (uint32_t)(Co / 16)) * gy, 16 * p.region);
+        for (int per_sm = 512 / p.cols; per_sm >= 1 && !found; --per_sm) {
+            long long budget = (long long)kSmemPerSM / per_sm - kSmemReserved;
+            if (budget > kSmemPerBlockMax) budget = kSmemPerBlockMax;
+            for (int ns = 4; ns >= 2; --ns) {
+                p.stages = ns;
+                if ((long long)wg_smem(p) <= budget) {
+                    found = true;
+                    resident = per_sm;
+                    break;
+                }
+            }
+        }
+    }
+    if (!found) return false;
+    p.nyb = (a.H + p.by - 1) / p.by;
+    const long long nkb = (long long)a.N * a.D * p.nyb;
+    if (nkb > 0x7FFFFFFFLL) return false;
+    const int by_blocks = Ci / 32;
+    long long npb = (long long)kWgWaves * resident * sm_count() / by_blocks;  // no partial last wave
+    if (npb < 1) npb = 1;
+    if (npb > nkb) npb = nkb;
+    p.kpb = (int)((nkb + npb - 1) / npb);
+    p.npb = (int)((nkb + p.kpb - 1) / p.kpb);
+    return by_blocks <= 65535;
+}
+
+// weight-gradient kernels with resident tiles, and the plan of the one a call runs under the current choice
+enum WgKernel { kWgPairs = 0, kWgDz = 1, kWgCopies = 2, kWgNone = -1 };
+static WgKernel wg_choose(const Act &a, int Ci, int Co, WgPlan &p) {
+    if (g_wgrad_algo == 0 && wg_copies_plan(a, Ci, Co, p)) return kWgCopies;
+    if (g_wgrad_algo != 3 && wg_dz_plan(a, Ci, Co, p)) return kWgDz;
+    return wg_plan(a, Ci, Co, p) ? kWgPairs : kWgNone;
+}
+
 static size_t wg_smem_request(const WgPlan &p) {
     size_t s = wg_smem(p);
     const int per_sm = 512 / p.cols;
@@ -1731,26 +1817,22 @@ static size_t wg_smem_request(const WgPlan &p) {
 
 // the weight-gradient partials of k_conv3_wgrad_res into part [npb][27 Ci][Co]
 static int conv3_wgrad_res(const void *x, int ldx, const void *dy, int ldy, float *part, float *bpart, const Act &a,
-                           int Ci, int Co, cudaStream_t s, const WgPlan &pl, bool dz_slots) {
+                           int Ci, int Co, cudaStream_t s, const WgPlan &pl, WgKernel kind) {
     CUtensorMap xmap, dymap;
-    const int box_c = dz_slots ? 8 : 16;
-    const CUtensorMapSwizzle swz = dz_slots ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_32B;
-    if (!act_map(&xmap, x, ldx, a, Ci, box_c, pl.pitch, dz_slots ? pl.by + 2 : pl.by, swz) ||
+    const int box_c = kind == kWgDz ? 8 : 16, lines = kind == kWgPairs ? pl.by : pl.by + 2;
+    const CUtensorMapSwizzle swz = kind == kWgDz ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_32B;
+    if (!act_map(&xmap, x, ldx, a, Ci, box_c, pl.pitch, lines, swz) ||
         !act_map(&dymap, dy, ldy, a, Co, box_c, pl.pitch, pl.by, swz))
         return 2;
     const size_t smem = wg_smem_request(pl);
-    static size_t attr[2] = {0, 0};
-    if (attr[dz_slots] < smem) {
-        if (cudaFuncSetAttribute(dz_slots ? k_conv3_wgrad_dz : k_conv3_wgrad_res,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-            return 2;
-        attr[dz_slots] = smem;
+    auto fn = kind == kWgPairs ? k_conv3_wgrad_res : kind == kWgDz ? k_conv3_wgrad_dz<false> : k_conv3_wgrad_dz<true>;
+    static size_t attr[3] = {0, 0, 0};
+    if (attr[kind] < smem) {
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 2;
+        attr[kind] = smem;
     }
     const dim3 grid((unsigned)pl.npb, (unsigned)((Ci / pl.ci_blk) * pl.ntile), 1);
-    if (dz_slots)
-        k_conv3_wgrad_dz<<<grid, RTHREADS, smem, s>>>(xmap, dymap, part, bpart, a, Ci, Co, pl);
-    else
-        k_conv3_wgrad_res<<<grid, RTHREADS, smem, s>>>(xmap, dymap, part, bpart, a, Ci, Co, pl);
+    fn<<<grid, RTHREADS, smem, s>>>(xmap, dymap, part, bpart, a, Ci, Co, pl);
     return cudaGetLastError() == cudaSuccess ? 0 : 2;
 }
 
@@ -1828,9 +1910,9 @@ int ws_conv3d_plan(int which, int N, int D, int H, int W, int Ci, int Co, long l
     } else {
         WgPlan pl;
         if (g_wgrad_algo == 1) return -1;
-        const bool dz = g_wgrad_algo != 3 && wg_dz_plan(a, Ci, Co, pl);
-        if (!dz && !wg_plan(a, Ci, Co, pl)) return -1;
-        const long long f[16] = {dz ? 1 : 0, pl.by, pl.nyb, pl.pitch, pl.ksteps, pl.J, pl.ci_blk, pl.ntile,
+        const WgKernel kind = wg_choose(a, Ci, Co, pl);
+        if (kind == kWgNone) return -1;
+        const long long f[16] = {kind, pl.by, pl.nyb, pl.pitch, pl.ksteps, pl.J, pl.ci_blk, pl.ntile,
                                  pl.npb, pl.kpb, pl.stages, pl.cols, pl.region, pl.stage_bytes,
                                  (long long)wg_smem_request(pl), (long long)(Ci / pl.ci_blk) * pl.ntile};
         for (; n < 16; ++n) v[n] = f[n];
@@ -1881,16 +1963,16 @@ int ws_conv3d_bwd_weight(const void *x, int ldx, const void *dy, int ldy, float 
     if (k == 3 && g_wgrad_algo != 1) {
         WgPlan pl;
         // Ci a multiple of 32 and Co <= 48: the dz-slot kernel (each X line loaded 3 times, not 9)
-        const bool dz_slots = g_wgrad_algo != 3 && wg_dz_plan(a, Ci, Co, pl);
-        if (dz_slots || wg_plan(a, Ci, Co, pl)) {
+        const WgKernel kind = wg_choose(a, Ci, Co, pl);
+        if (kind != kWgNone) {
             // the kernel sums the bias gradient too when it has a free slot for a row of ones
-            const bool fold = db && (dz_slots || pl.J * pl.ntile > 9);
+            const bool fold = db && (kind != kWgPairs || pl.J * pl.ntile > 9);
             const size_t wpart = (size_t)pl.npb * 27 * Ci * Co;
             const size_t bparts = fold ? (size_t)pl.npb : (size_t)nbb;
             float *ws_buf = grad_workspace((wpart + bparts * Co) * sizeof(float), s);
             if (!ws_buf) return 2;
             float *bpart = ws_buf + wpart;
-            const int rc = conv3_wgrad_res(x, ldx, dy, ldy, ws_buf, fold ? bpart : nullptr, a, Ci, Co, s, pl, dz_slots);
+            const int rc = conv3_wgrad_res(x, ldx, dy, ldy, ws_buf, fold ? bpart : nullptr, a, Ci, Co, s, pl, kind);
             if (rc) return rc;
             if (db && !fold) {
                 const dim3 g2((unsigned)nbb, (unsigned)((Co + 31) / 32), 1);

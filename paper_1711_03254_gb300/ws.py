@@ -92,8 +92,8 @@ def ws_conv3d_fwd_algo(algo: str) -> str:
 
 def ws_conv3d_bwd_weight_algo(algo: str) -> str:
     """Weight-gradient kernel of later ws_conv3d_bwd_weight calls: "auto",
-    "gather", "resident" or "pairs" (resident, tap-pair rows only); returns
-    the previous choice."""
+    "gather", "resident" (resident tiles without copies of dy) or "pairs"
+    (resident, tap-pair rows only); returns the previous choice."""
     names = ("auto", "gather", "resident", "pairs")
     prev = _lib().ws_conv3d_bwd_weight_algo(names.index(algo))
     if prev < 0:

@@ -196,3 +196,33 @@ def test_mse_and_adam(env):
     wr = w - 1e-3 * mr / (np.sqrt(vr) + 1e-8)
     assert np.allclose(wt.cpu().numpy(), wr, rtol=1e-5, atol=1e-7)
     assert np.allclose(wb.float().cpu().numpy(), wr, rtol=1e-2, atol=1e-3)
+
+
+@pytest.mark.parametrize("shape,Ci,Co", [((1, 1, 1, 1), 32, 16), ((2, 3, 7, 5), 32, 48), ((1, 4, 13, 64), 64, 32),
+                                         ((2, 2, 9, 30), 96, 16), ((1, 3, 5, 126), 32, 32), ((1, 2, 3, 254), 32, 16),
+                                         ((3, 5, 16, 16), 32, 32), ((1, 2, 3, 130), 32, 48)])
+def test_weight_gradient_with_copies(env, shape, Ci, Co):
+    """The automatic weight gradient (three copies of dY side by side where
+    Ci is a multiple of 32 and Co <= 48) at one and several lines per K-block,
+    K-blocks that are and are not whole K-steps, ragged last K-blocks, and widths
+    where no such plan fits, from channel slices, against the oracle."""
+    torch, ws, conv = env
+    rng = np.random.default_rng(sum(shape) + Ci + Co)
+    x = _bf16_round(torch, rng.standard_normal(shape + (Ci,)))
+    dy = _bf16_round(torch, rng.standard_normal(shape + (Co,)))
+    xb = torch.zeros(shape + (Ci + 16,), dtype=torch.bfloat16, device="cuda")
+    xb[..., 8:8 + Ci] = torch.from_numpy(x).cuda()
+    yb = torch.full(shape + (Co + 8,), 7.0, dtype=torch.bfloat16, device="cuda")
+    yb[..., 8:] = torch.from_numpy(dy).cuda()
+    dw = torch.ones((Co, 3, 3, 3, Ci), device="cuda")
+    db = torch.ones(Co, device="cuda")
+    prev = ws.ws_conv3d_bwd_weight_algo("auto")
+    try:
+        ws.ws_conv3d_bwd_weight(xb[..., 8:8 + Ci], yb[..., 8:], dw, db, 3)
+    finally:
+        ws.ws_conv3d_bwd_weight_algo(prev)
+    assert ws.ws_tc_status() == 0
+    ref_w, ref_b = conv.conv3d_bwd_weight(x, dy, 3)
+    # FP32 accumulation over the positions, as for the other kernels
+    assert _rel(dw.cpu().numpy() - 1.0, ref_w) < 2e-5
+    assert _rel(db.cpu().numpy() - 1.0, ref_b) < 2e-5
