@@ -40,8 +40,9 @@ extern "C" {
  *    of the plane are shifted views of that tile.  For Co >= 64 or Ci = 16,
  *    where two accumulator buffers fit the tensor memory, one persistent
  *    block per SM strides over the tiles (the epilogue of a tile overlapping
- *    the next tile's MMAs); otherwise each block computes one tile.  Both give
- *    the same bits;
+ *    the next tile's MMAs); otherwise each block computes one tile.  The
+ *    automatic choice gives small grids fewer lines per tile, or blocks that
+ *    compute a part of the output channels.  All give the same bits;
  *  - gathered tiles (k = 1, and k = 3 where no resident plan fits): 128
  *    positions per block, each tap's rows gathered with 16-byte copies.
  * Additional argument rules: Co <= 256, y 16-byte aligned, ldy a multiple of
@@ -52,8 +53,9 @@ int ws_conv3d_fwd(const void *x, int ldx, const void *w, const float *bias, void
                   int D, int H, int W, int Ci, int Co, int k, int relu, void *stream);
 
 /* Selects the forward kernel of later ws_conv3d_fwd calls (process-wide):
- * 0 automatic (resident tiles where a plan fits, else gathered), 1 gathered
- * tiles always, 2 resident tiles always for k = 3, 3 as 2 but one block per
+ * 0 automatic (resident tiles where a plan fits, split for small grids, else
+ * gathered), 1 gathered tiles always, 2 resident tiles always for k = 3 (every
+ * tile with all output channels), 3 as 2 but one block per
  * tile (never the persistent kernel), 4 as 2 but persistent wherever its
  * buffers fit.  Returns the previous choice, or -1 for an unknown value
  * (nothing changes). */

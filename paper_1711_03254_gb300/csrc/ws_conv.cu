@@ -121,6 +121,80 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity) {
     return false;
 }
 
+// Epilogue of one accumulator row per thread: Co columns from tensor memory at
+// taddr, plus bias (in shared memory; NULL: none), ReLU, to row `dst` of the
+// output.  Two loads of 16 columns are in flight at a time.  The bias comes from
+// shared memory, four columns a load: read from global memory, a scalar at a
+// time, it made the persistent kernel's epilogue longer than the MMAs it hides
+// behind (64^3 32->96, batch 4: 324 us with bias, 216 without).
+template <bool OUT_F32>
+__device__ __forceinline__ void epilogue_row(uint32_t taddr, int Co, bool valid, void *dst, const float *sbias,
+                                             int relu) {
+    for (int c0 = 0; c0 < Co; c0 += 32) {
+        const int halves = c0 + 16 < Co ? 2 : 1;
+        uint32_t v[2][16];
+        __syncwarp();
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            if (h < halves)
+                asm volatile(
+                    "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
+                    "[%16];\n"
+                    : "=r"(v[h][0]), "=r"(v[h][1]), "=r"(v[h][2]), "=r"(v[h][3]), "=r"(v[h][4]), "=r"(v[h][5]),
+                      "=r"(v[h][6]), "=r"(v[h][7]), "=r"(v[h][8]), "=r"(v[h][9]), "=r"(v[h][10]), "=r"(v[h][11]),
+                      "=r"(v[h][12]), "=r"(v[h][13]), "=r"(v[h][14]), "=r"(v[h][15])
+                    : "r"(taddr + (uint32_t)(c0 + 16 * h)));
+        asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (h >= halves || !valid) continue;
+            const int c = c0 + 16 * h;
+            float o[16];
+#pragma unroll
+            for (int e = 0; e < 16; ++e) o[e] = __uint_as_float(v[h][e]);
+            if (sbias) {
+#pragma unroll
+                for (int e = 0; e < 16; e += 4) {
+                    const float4 b = *reinterpret_cast<const float4 *>(sbias + c + e);
+                    o[e] += b.x, o[e + 1] += b.y, o[e + 2] += b.z, o[e + 3] += b.w;
+                }
+            }
+            if (relu) {
+#pragma unroll
+                for (int e = 0; e < 16; ++e) o[e] = fmaxf(o[e], 0.f);
+            }
+            if (OUT_F32) {
+                float4 *d = reinterpret_cast<float4 *>((float *)dst + c);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) d[e] = make_float4(o[4 * e], o[4 * e + 1], o[4 * e + 2], o[4 * e + 3]);
+            } else {
+                uint4 *d = reinterpret_cast<uint4 *>((bf16 *)dst + c);
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    __nv_bfloat162 b[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) b[k] = __floats2bfloat162_rn(o[8 * e + 2 * k], o[8 * e + 2 * k + 1]);
+                    uint4 u;
+                    u.x = *reinterpret_cast<uint32_t *>(&b[0]);
+                    u.y = *reinterpret_cast<uint32_t *>(&b[1]);
+                    u.z = *reinterpret_cast<uint32_t *>(&b[2]);
+                    u.w = *reinterpret_cast<uint32_t *>(&b[3]);
+                    d[e] = u;
+                }
+            }
+        }
+    }
+}
+
+constexpr int kMaxCo = 256;  // output channels of the forward kernels
+// the bias to shared memory (a block barrier follows); NULL stays NULL
+template <int THREADS>
+__device__ __forceinline__ const float *stage_bias(float *sbias, const float *bias, int Co) {
+    if (!bias) return nullptr;
+    for (int c = threadIdx.x; c < Co; c += THREADS) sbias[c] = bias[c];
+    return sbias;
+}
+
 template <bool OUT_F32>
 __global__ void __launch_bounds__(TTHREADS) k_conv_fwd_tc(const bf16 *__restrict__ X, int ldx,
                                                          const bf16 *__restrict__ Wt, const float *__restrict__ bias,
@@ -139,6 +213,8 @@ __global__ void __launch_bounds__(TTHREADS) k_conv_fwd_tc(const bf16 *__restrict
     const int r = k / 2, KV = k * k * k, cchunks = Ci / 16;
     const int nkc = KV * cchunks, nkb = (nkc + TKC - 1) / TKC;
 
+    __shared__ __align__(16) float sbias[kMaxCo];
+    const float *sb_ptr = stage_bias<TTHREADS>(sbias, bias, BN);
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tslot)),
                      "r"(tmem_cols));
@@ -162,6 +238,14 @@ __global__ void __launch_bounds__(TTHREADS) k_conv_fwd_tc(const bf16 *__restrict
     for (int j = 0; j < 2; ++j) {
         const long long p = m0 + j * 64 + (tid >> 1);
         prow[j] = p < P;
+        if (P <= 0x7FFFFFFFLL) {  // 32-bit divisions where they do
+            uint32_t q = prow[j] ? (uint32_t)p : 0u;
+            px[j] = (int)(q % (uint32_t)a.W); q /= (uint32_t)a.W;
+            py[j] = (int)(q % (uint32_t)a.H); q /= (uint32_t)a.H;
+            pz[j] = (int)(q % (uint32_t)a.D); q /= (uint32_t)a.D;
+            pn[j] = (int)q;
+            continue;
+        }
         long long q = prow[j] ? p : 0;
         px[j] = (int)(q % a.W); q /= a.W;
         py[j] = (int)(q % a.H); q /= a.H;
@@ -244,37 +328,8 @@ __global__ void __launch_bounds__(TTHREADS) k_conv_fwd_tc(const bf16 *__restrict
     if (ok_run) {
         // epilogue: warp w owns accumulator rows (TMEM lanes) 32 w .. 32 w + 31
         const long long row = m0 + warp * 32 + lane;
-        for (int c0 = 0; c0 < BN; c0 += 16) {
-            uint32_t v[16];
-            const uint32_t addr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
-            asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
-                "[%16];\n"
-                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                  "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
-                  "=r"(v[15])
-                : "r"(addr));
-            asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::);
-            if (row < P) {
-                float o[16];
-#pragma unroll
-                for (int e = 0; e < 16; ++e) {
-                    float x = __uint_as_float(v[e]);
-                    if (bias) x += bias[c0 + e];
-                    if (relu) x = fmaxf(x, 0.f);
-                    o[e] = x;
-                }
-                if (OUT_F32) {
-                    float4 *dst = reinterpret_cast<float4 *>((float *)Y + row * ldy + c0);
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) dst[e] = make_float4(o[4 * e], o[4 * e + 1], o[4 * e + 2], o[4 * e + 3]);
-                } else {
-                    __nv_bfloat162 *dst = reinterpret_cast<__nv_bfloat162 *>((bf16 *)Y + row * ldy + c0);
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) dst[e] = __floats2bfloat162_rn(o[2 * e], o[2 * e + 1]);
-                }
-            }
-        }
+        void *dst = OUT_F32 ? (void *)((float *)Y + row * ldy) : (void *)((bf16 *)Y + row * ldy);
+        epilogue_row<OUT_F32>(tmem + ((uint32_t)(warp * 32) << 16), BN, row < P, dst, sb_ptr, relu);
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::);
     __syncthreads();
@@ -301,6 +356,9 @@ __global__ void __launch_bounds__(TTHREADS) k_conv_fwd_tc(const bf16 *__restrict
 // matrices, so any 16-byte start is a valid tile; the two K halves of a chunk
 // are separate boxes one leading byte offset apart.  The weights of the 9 taps
 // of (c, dz) arrive by TMA as [tap][K half][Co rows] tiles.
+//
+// With nco > 1 a block computes Co of the nco x Co output channels (small grids,
+// see small_grid_plan).
 //
 // Roles: thread 0 issues the TMA loads into a ring of stages, thread 32
 // issues the MMAs (M = 128 rows per tile, N = Co, K = 16) into one
@@ -337,7 +395,7 @@ template <bool OUT_F32>
 __global__ void __launch_bounds__(RTHREADS) k_conv3_fwd_res(const __grid_constant__ CUtensorMap xmap,
                                                            const __grid_constant__ CUtensorMap wmap,
                                                            const float *__restrict__ bias, void *__restrict__ Y,
-                                                           int ldy, Act a, int Ci, int Co, int relu, ResPlan pl) {
+                                                           int ldy, Act a, int Ci, int Co, int nco, int relu, ResPlan pl) {
     extern __shared__ __align__(128) unsigned char sm_raw[];
     unsigned char *sm = sm_raw + ((1024u - (smem_u32(sm_raw) & 1023u)) & 1023u);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -348,8 +406,9 @@ __global__ void __launch_bounds__(RTHREADS) k_conv3_fwd_res(const __grid_constan
     uint32_t *tslot = reinterpret_cast<uint32_t *>(done + 1);
     int *abort_flag = reinterpret_cast<int *>(tslot + 1);
 
-    // the tile: lines y0 .. y0 + lt - 1 of plane z of sample n
-    const int yt = blockIdx.x % pl.nyt, zn = blockIdx.x / pl.nyt;
+    // the tile: lines y0 .. y0 + lt - 1 of plane z of sample n, output channels co0 .. co0 + Co - 1
+    const int tile = (int)blockIdx.x / nco, co0 = ((int)blockIdx.x - tile * nco) * Co;
+    const int yt = tile % pl.nyt, zn = tile / pl.nyt;
     const int z = zn % a.D, n = zn / a.D;
     const int y0 = yt * pl.by, lt = min(pl.by, a.H - y0);
     const int nt = ((lt - 1) * pl.pitch + a.W + 127) / 128;
@@ -389,7 +448,7 @@ __global__ void __launch_bounds__(RTHREADS) k_conv3_fwd_res(const __grid_constan
                          : "memory");
             const uint32_t sa = base + (uint32_t)st * pl.stage_bytes, sb = sa + 2 * pl.a_half;
             tma_load_5d(sa, &xmap, c * 16, -1, y0 - 1, z + dz - 1, n, fb);
-            tma_load_3d(sb, &wmap, c * 16, 0, dz * 9, fb);
+            tma_load_3d(sb, &wmap, c * 16, co0, dz * 9, fb);
             issued = s + 1;
         }
         // wait for the loads still in flight (the last phase issued on each stage)
@@ -439,6 +498,9 @@ __global__ void __launch_bounds__(RTHREADS) k_conv3_fwd_res(const __grid_constan
     const bool ok_run = __syncthreads_and(okw) && *(volatile int *)abort_flag == 0;
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
 
+    // the MMAs are done with the stages: the bias goes where the first one was
+    const float *sb_ptr = ok_run ? stage_bias<RTHREADS>(reinterpret_cast<float *>(sm), bias ? bias + co0 : nullptr, Co) : nullptr;
+    __syncthreads();
     if (ok_run) {
         // epilogue: warp w owns accumulator rows (TMEM lanes) 32 w .. 32 w + 31 of every tile
         for (int j = 0; j < nt; ++j) {
@@ -446,49 +508,9 @@ __global__ void __launch_bounds__(RTHREADS) k_conv3_fwd_res(const __grid_constan
             const int line = q / pl.pitch, x = q - line * pl.pitch;
             const bool valid = x < a.W && line < lt;
             const long long row = (((long long)n * a.D + z) * a.H + y0 + line) * a.W + x;
-            for (int c0 = 0; c0 < Co; c0 += 16) {
-                uint32_t v[16];
-                const uint32_t addr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(j * Co + c0);
-                asm volatile(
-                    "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
-                    "[%16];\n"
-                    : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                      "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
-                      "=r"(v[15])
-                    : "r"(addr));
-                asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::);
-                if (valid) {
-                    float o[16];
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        float xv = __uint_as_float(v[e]);
-                        if (bias) xv += bias[c0 + e];
-                        if (relu) xv = fmaxf(xv, 0.f);
-                        o[e] = xv;
-                    }
-                    if (OUT_F32) {
-                        float4 *dst = reinterpret_cast<float4 *>((float *)Y + row * ldy + c0);
-#pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            dst[e] = make_float4(o[4 * e], o[4 * e + 1], o[4 * e + 2], o[4 * e + 3]);
-                    } else {
-                        uint4 *dst = reinterpret_cast<uint4 *>((bf16 *)Y + row * ldy + c0);
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            uint4 u;
-                            __nv_bfloat162 h0 = __floats2bfloat162_rn(o[8 * e], o[8 * e + 1]);
-                            __nv_bfloat162 h1 = __floats2bfloat162_rn(o[8 * e + 2], o[8 * e + 3]);
-                            __nv_bfloat162 h2 = __floats2bfloat162_rn(o[8 * e + 4], o[8 * e + 5]);
-                            __nv_bfloat162 h3 = __floats2bfloat162_rn(o[8 * e + 6], o[8 * e + 7]);
-                            u.x = *reinterpret_cast<uint32_t *>(&h0);
-                            u.y = *reinterpret_cast<uint32_t *>(&h1);
-                            u.z = *reinterpret_cast<uint32_t *>(&h2);
-                            u.w = *reinterpret_cast<uint32_t *>(&h3);
-                            dst[e] = u;
-                        }
-                    }
-                }
-            }
+            void *dst = OUT_F32 ? (void *)((float *)Y + row * ldy + co0) : (void *)((bf16 *)Y + row * ldy + co0);
+            epilogue_row<OUT_F32>(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(j * Co), Co, valid, dst, sb_ptr,
+                                  relu);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::);
@@ -554,6 +576,8 @@ __global__ void __launch_bounds__(PTHREADS, 1) k_conv3_fwd_pers(const __grid_con
     uint32_t *tslot = reinterpret_cast<uint32_t *>(done + 1);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tslot + 1);
 
+    float *sbias = reinterpret_cast<float *>((reinterpret_cast<uintptr_t>(tslot + 2) + 15) & ~(uintptr_t)15);
+    const float *sb_ptr = stage_bias<PTHREADS>(sbias, bias, Co);
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tslot)),
                      "r"(pl.cols));
@@ -672,49 +696,10 @@ __global__ void __launch_bounds__(PTHREADS, 1) k_conv3_fwd_pers(const __grid_con
                 const int line = q / pl.pitch, x = q - line * pl.pitch;
                 const bool valid = x < a.W && line < r.lt;
                 const long long row = (((long long)r.n * a.D + r.z) * a.H + r.y0 + line) * a.W + x;
-                for (int c0 = 0; c0 < Co; c0 += 16) {
-                    uint32_t v[16];
-                    const uint32_t addr =
-                        tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)buf * buf_cols + (uint32_t)(j * Co + c0);
-                    asm volatile(
-                        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
-                        "%15}, [%16];\n"
-                        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-                          "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
-                          "=r"(v[14]), "=r"(v[15])
-                        : "r"(addr));
-                    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::);
-                    if (valid) {
-                        float o[16];
-#pragma unroll
-                        for (int e = 0; e < 16; ++e) {
-                            float xv = __uint_as_float(v[e]);
-                            if (bias) xv += bias[c0 + e];
-                            if (relu) xv = fmaxf(xv, 0.f);
-                            o[e] = xv;
-                        }
-                        if (OUT_F32) {
-                            float4 *dst = reinterpret_cast<float4 *>((float *)Y + row * ldy + c0);
-#pragma unroll
-                            for (int e = 0; e < 4; ++e)
-                                dst[e] = make_float4(o[4 * e], o[4 * e + 1], o[4 * e + 2], o[4 * e + 3]);
-                        } else {
-                            uint4 *dst = reinterpret_cast<uint4 *>((bf16 *)Y + row * ldy + c0);
-#pragma unroll
-                            for (int e = 0; e < 2; ++e) {
-                                __nv_bfloat162 h[4];
-#pragma unroll
-                                for (int k = 0; k < 4; ++k) h[k] = __floats2bfloat162_rn(o[8 * e + 2 * k], o[8 * e + 2 * k + 1]);
-                                uint4 u;
-                                u.x = *reinterpret_cast<uint32_t *>(&h[0]);
-                                u.y = *reinterpret_cast<uint32_t *>(&h[1]);
-                                u.z = *reinterpret_cast<uint32_t *>(&h[2]);
-                                u.w = *reinterpret_cast<uint32_t *>(&h[3]);
-                                dst[e] = u;
-                            }
-                        }
-                    }
-                }
+                void *dst = OUT_F32 ? (void *)((float *)Y + row * ldy) : (void *)((bf16 *)Y + row * ldy);
+                epilogue_row<OUT_F32>(
+                    tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)buf * buf_cols + (uint32_t)(j * Co), Co, valid,
+                    dst, sb_ptr, relu);
             }
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::);
             __syncwarp();
@@ -1552,7 +1537,9 @@ static bool act_map(CUtensorMap *map, const void *t, int ld, const Act &a, int C
 // pair within the 512 columns), one block per SM, the most stages (2 ..
 // kPersStages) that fit.  False where the buffers do not fit.
 constexpr int kPersStages = 4;
-static size_t pers_smem(const ResPlan &p) { return (size_t)p.stages * p.stage_bytes + 1024 + 8 * (2 * p.stages + 5) + 16; }
+static size_t pers_smem(const ResPlan &p) {
+    return (size_t)p.stages * p.stage_bytes + 1024 + 8 * (2 * p.stages + 5) + 16 + 16 + kMaxCo * sizeof(float);
+}
 static bool pers_plan(const ResPlan &res, int Co, ResPlan &p, uint32_t &buf_cols) {
     p = res;
     buf_cols = 32;
@@ -1565,17 +1552,108 @@ static bool pers_plan(const ResPlan &res, int Co, ResPlan &p, uint32_t &buf_cols
     return false;
 }
 
-// The persistent forward kernel where it measured faster (U-Net layers at 64^3,
-// 32^3, 16^3, batch 4): Co >= 64 (32^3 64->64: 517 against 466 TFLOP/s) and
-// 16-channel inputs (3 K-steps a tile; 64^3 16->32: 381 against 321); one
-// block per tile for narrower outputs of wider inputs (64^3 96->32: 617
-// against 478, 32->32: 440 against 433).
+// The persistent forward kernel where it measured faster (U-Net layers, batch
+// 4, us): Co >= 64 (32^3 64->64: 50.1 against 52.8, 32->64: 29.1 against 34.0) and
+// 16-channel inputs; one block per tile for narrower outputs of wider inputs
+// (64^3 96->32: 252 against 366, 32->32: 103 against 134).  The automatic choice
+// also runs one block per tile where there is at most one tile per SM and
+// nothing to overlap (16^3 224->96: 38.3 against 43.1, one sample of 32^3 64->64: 18.5
+// against 20.3).
 static bool want_persistent(int Ci, int Co) {
     return g_fwd_algo == 4 || (g_fwd_algo != 3 && (Co >= 64 || Ci <= 16));
 }
 
+// Small grids (automatic choice): a plan that leaves SMs idle, or one block per
+// SM where two would share its tensor core, is replaced by one with fewer lines
+// per tile, more resident blocks or the output channels split over nco blocks,
+// when a model of the kernel's time says so by more than 10 %.  The model, in
+// SM clocks, from measurements on GB300 with loads or MMAs left out: an M128 K16
+// MMA takes about 43 + 0.65 N (at least 105 when one block is alone on its SM,
+// because consecutive MMAs on one accumulator wait for each other), TMA 1.5
+// per 32-byte row, both shared by the blocks of an SM, 3000 per round of
+// resident blocks for the start and the epilogue.  Neither choice changes the
+// order of any sum, so the bits stay.  us per call, before and after: 8^3
+// 128->128 20.6, 16.5; 16^3 96->96 21.7, 13.6; 224->96 42.9, 26.6; batch 4, 32^3
+// 160->64 114, 94; 64->64 50, 45.  (At 3 % instead of 10 it also moved 64^3 32->32
+// from 11 lines to 13: 111 us against 103.)
+struct GridCost {
+    double clocks;
+    int per_sm;
+};
+static GridCost grid_cost(const Act &a, int Ci, int N, int nco, int by, int nt, int pitch, int per_sm, bool persistent) {
+    const long long blocks = (long long)a.N * a.D * ((a.H + by - 1) / by) * nco;
+    const long long m = (blocks + sm_count() - 1) / sm_count();  // blocks of the busiest SM
+    const bool alone = m < 2 || persistent || per_sm < 2;
+    const double mma = 9.0 * nt * (alone ? std::max(105.0, 59.0 + 0.65 * N) : 43.0 + 0.65 * N);
+    const double tma = 1.5 * ((by + 2) * pitch + 9.0 * N);
+    const long long rounds = persistent ? 1 : (m + per_sm - 1) / per_sm;
+    return {(double)m * (Ci / 16) * 3.0 * std::max(mma, tma) + 3000.0 * (double)rounds, per_sm};
+}
+static bool small_grid_plan(const Act &a, int Ci, int Co, const ResPlan &base, bool persistent, ResPlan &out,
+                            int &nco_out) {
+    const long long base_blocks = (long long)a.N * a.D * base.nyt;
+    if (base_blocks > 12LL * sm_count()) return false;
+    const int pitch = base.pitch;
+    double best = 0.9 * grid_cost(a, Ci, Co, 1, base.by, base.ntiles, pitch, persistent ? 1 : base.per_sm, persistent).clocks;
+    bool found = false;
+    for (int nco : {1, 2, 3, 4, 6, 8}) {
+        if (Co % (16 * nco)) continue;
+        const int N = Co / nco;
+        for (int want = 1; want * N <= 512; ++want) {
+            int by = (128 * want - a.W) / pitch + 1;
+            if (128 * want < a.W || by < 1) continue;
+            by = std::min(std::min(by, a.H), 254);
+            const int nyt = (a.H + by - 1) / by;
+            by = (a.H + nyt - 1) / nyt;  // the same tiles per plane, evenly
+            ResPlan p;
+            p.by = by;
+            p.nyt = (a.H + by - 1) / by;
+            p.pitch = pitch;
+            p.ntiles = res_tiles(by, pitch, a.W);
+            p.cols = 32;
+            while (p.cols < p.ntiles * N) p.cols *= 2;
+            const int R = (std::max(128 * p.ntiles + 2 * pitch + 2, (by + 2) * pitch) + 7) / 8 * 8;
+            p.a_half = (uint32_t)R * 16u;
+            p.stage_bytes = 2 * p.a_half + 18u * (uint32_t)N * 16u;
+            p.tx_bytes = 2u * (uint32_t)((by + 2) * pitch) * 16u + 18u * (uint32_t)N * 16u;
+            const long long blocks = (long long)a.N * a.D * p.nyt * nco, m = (blocks + sm_count() - 1) / sm_count();
+            // as many resident blocks as the busiest SM has work for, 2 .. 8 stages each
+            p.per_sm = (int)std::min<long long>(std::min<long long>(m, 512 / p.cols), 4);
+            for (p.stages = 0; p.per_sm >= 1 && !p.stages; p.per_sm -= p.stages ? 0 : 1)
+                for (int ns = 8; ns >= 2 && !p.stages; --ns) {
+                    ResPlan q = p;
+                    q.stages = ns;
+                    const long long budget =
+                        std::min((long long)kSmemPerSM / p.per_sm - kSmemReserved, (long long)kSmemPerBlockMax);
+                    if ((long long)res_smem(q) <= budget) p.stages = ns;
+                }
+            if (!p.stages) continue;
+            const double c = grid_cost(a, Ci, N, nco, by, p.ntiles, pitch, p.per_sm, false).clocks;
+            if (c < best) {
+                best = c;
+                out = p;
+                nco_out = nco;
+                found = true;
+            }
+        }
+    }
+    return found;
+}
+
 static int conv3_fwd_res(const void *x, int ldx, const void *w, const float *bias, void *y, int ldy, int y_f32,
-                         const Act &a, int Ci, int Co, int relu, cudaStream_t s, const ResPlan &pl) {
+                         const Act &a, int Ci, int Co, int relu, cudaStream_t s, ResPlan pl) {
+    ResPlan pp;
+    uint32_t buf_cols = 0;
+    bool persistent = want_persistent(Ci, Co) && pers_plan(pl, Co, pp, buf_cols);
+    int nco = 1;
+    if (g_fwd_algo == 0) {
+        ResPlan sp;
+        persistent = persistent && (long long)a.N * a.D * pl.nyt > sm_count();
+        if (small_grid_plan(a, Ci, Co, pl, persistent, sp, nco)) {
+            pl = sp;
+            persistent = false;
+        }
+    }
     EncodeTiledFn enc = encode_tiled();
     CUtensorMap xmap, wmap;
     if (!enc || !act_map(&xmap, x, ldx, a, Ci, 16, pl.pitch, pl.by + 2, CU_TENSOR_MAP_SWIZZLE_32B)) return 2;
@@ -1583,7 +1661,7 @@ static int conv3_fwd_res(const void *x, int ldx, const void *w, const float *bia
     const cuuint32_t ones[3] = {1, 1, 1};
     const cuuint64_t wdim[3] = {(cuuint64_t)Ci, (cuuint64_t)Co, 27};
     const cuuint64_t wstr[2] = {(cuuint64_t)Ci * 2 * 27, (cuuint64_t)Ci * 2};
-    const cuuint32_t wbox[3] = {16, (cuuint32_t)Co, 9};
+    const cuuint32_t wbox[3] = {16, (cuuint32_t)(Co / nco), 9};
     if (enc(&wmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(w), wdim, wstr, wbox, ones,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
@@ -1599,11 +1677,9 @@ static int conv3_fwd_res(const void *x, int ldx, const void *w, const float *bia
         if (e != cudaSuccess) return 2;
         attr[which] = smem;
     }
-    const long long blocks = (long long)a.N * a.D * pl.nyt;
+    const long long blocks = (long long)a.N * a.D * pl.nyt * nco;
     if (blocks > 0x7FFFFFFFLL) return 1;
-    ResPlan pp;
-    uint32_t buf_cols = 0;
-    if (want_persistent(Ci, Co) && pers_plan(pl, Co, pp, buf_cols)) {
+    if (persistent) {
         // one persistent block per SM (at most one per tile)
         const size_t psmem = std::max(pers_smem(pp), (size_t)kSmemPerSM / 2 - kSmemReserved + 16);
         static size_t pattr[2] = {0, 0};
@@ -1625,9 +1701,11 @@ static int conv3_fwd_res(const void *x, int ldx, const void *w, const float *bia
         return cudaGetLastError() == cudaSuccess ? 0 : 2;
     }
     if (y_f32)
-        k_conv3_fwd_res<true><<<(unsigned)blocks, RTHREADS, smem, s>>>(xmap, wmap, bias, y, ldy, a, Ci, Co, relu, pl);
+        k_conv3_fwd_res<true><<<(unsigned)blocks, RTHREADS, smem, s>>>(xmap, wmap, bias, y, ldy, a, Ci, Co / nco, nco,
+                                                                       relu, pl);
     else
-        k_conv3_fwd_res<false><<<(unsigned)blocks, RTHREADS, smem, s>>>(xmap, wmap, bias, y, ldy, a, Ci, Co, relu, pl);
+        k_conv3_fwd_res<false><<<(unsigned)blocks, RTHREADS, smem, s>>>(xmap, wmap, bias, y, ldy, a, Ci, Co / nco, nco,
+                                                                        relu, pl);
     return cudaGetLastError() == cudaSuccess ? 0 : 2;
 }
 
@@ -1898,13 +1976,20 @@ int ws_conv3d_plan(int which, int N, int D, int H, int W, int Ci, int Co, long l
         uint32_t buf_cols = 0;
         if (g_fwd_algo == 1 || !res_plan(W, H, Co, pl)) return -1;
         const long long tiles = (long long)N * D * pl.nyt;
-        const bool pers = want_persistent(Ci, Co) && pers_plan(pl, Co, pp, buf_cols);
+        bool pers = want_persistent(Ci, Co) && pers_plan(pl, Co, pp, buf_cols);
+        ResPlan sp;
+        int nco = 1;
+        if (g_fwd_algo == 0) pers = pers && tiles > sm_count();
+        if (g_fwd_algo == 0 && small_grid_plan(a, Ci, Co, pl, pers, sp, nco)) {
+            pl = sp;
+            pers = false;
+        }
         const ResPlan &q = pers ? pp : pl;
         const size_t smem = pers ? std::max(pers_smem(pp), (size_t)kSmemPerSM / 2 - kSmemReserved + 16)
                                  : res_smem_request(pl);
         const long long f[14] = {pers ? 1 : 0, q.by, q.nyt, q.pitch, q.ntiles, q.stages, q.cols, q.per_sm,
                                  q.a_half, q.stage_bytes, q.tx_bytes, (long long)smem,
-                                 pers ? std::min<long long>(tiles, sm_count()) : tiles,
+                                 pers ? std::min<long long>(tiles, sm_count()) : (long long)N * D * pl.nyt * nco,
                                  pers ? (long long)buf_cols : 0};
         for (; n < 14; ++n) v[n] = f[n];
     } else {

@@ -226,3 +226,32 @@ def test_weight_gradient_with_copies(env, shape, Ci, Co):
     # FP32 accumulation over the positions, as for the other kernels
     assert _rel(dw.cpu().numpy() - 1.0, ref_w) < 2e-5
     assert _rel(db.cpu().numpy() - 1.0, ref_b) < 2e-5
+
+
+@pytest.mark.parametrize("shape,Ci,Co", [((1, 8, 8, 8), 128, 128), ((1, 16, 16, 16), 96, 96), ((2, 14, 19, 23), 96, 128),
+                                         ((1, 5, 33, 30), 64, 48), ((1, 3, 7, 130), 16, 160), ((1, 1, 1, 1), 16, 16),
+                                         ((1, 2, 50, 12), 32, 256), ((3, 9, 40, 16), 32, 32)])
+def test_small_grids_keep_the_bits(env, shape, Ci, Co):
+    """The automatic forward choice splits small grids over fewer lines or over
+    blocks of output channels; every output equals the unsplit kernel's, with
+    and without bias and ReLU, in FP32 and BF16, into channel slices."""
+    torch, ws, _ = env
+    g = torch.Generator(device="cuda").manual_seed(Ci + Co)
+    x = torch.randn(shape + (Ci,), generator=g, device="cuda").to(torch.bfloat16)
+    w = (torch.randn((Co, 3, 3, 3, Ci), generator=g, device="cuda") * 0.1).to(torch.bfloat16)
+    b = torch.randn(Co, generator=g, device="cuda")
+    out = []
+    prev = ws.ws_conv3d_fwd_algo("auto")
+    try:
+        for algo in ("auto", "pertile"):
+            ws.ws_conv3d_fwd_algo(algo)
+            y = torch.full(shape + (Co + 8,), 3.0, dtype=torch.bfloat16, device="cuda")
+            z = torch.full(shape + (Co + 4,), 3.0, dtype=torch.float32, device="cuda")
+            ws.ws_conv3d_fwd(x, w, b, y[..., 8:], True)
+            ws.ws_conv3d_fwd(x, w, None, z[..., :Co], False)
+            out.append((y, z))
+    finally:
+        ws.ws_conv3d_fwd_algo(prev)
+    assert ws.ws_tc_status() == 0
+    for p, q in zip(*out):
+        assert torch.equal(p, q)
