@@ -8,17 +8,17 @@
 
 namespace lbm {
 
-// Occupancy, measured on GB300 (256^3 packed spheres, ms per update).  The
-// update runs 128-thread blocks, 6 per SM for the FP32 and 16-bit storages
-// (80 registers, no spills) and 4 for FP64: FP16 0.297 against 0.317 at 5 and
-// 0.310 at 7 (72 registers, spilling), 256-thread blocks 3 per SM 0.322; FP32
-// 0.380 against 0.401 at 5, 0.415 at 7 and 0.441 at 4; FP64 the same at 3 to 5.
-// The psi pass runs 256-thread blocks, 6 per SM (40 registers): 16-bit
-// storage 0.139 ms against 0.159 at 4 and 0.192 at 3 per SM (5 and 8: 0.139),
-// and 0.163 for a persistent variant that prefetched each thread's next cell
-// with cp.async; FP32 0.186 against 0.218 at 3 per SM.
-constexpr int kPsiThreads = 256, kPsiBlocks = 6, kCollideThreads = 128;
-template <class S> constexpr int collide_min_blocks() { return sizeof(S) == 2 ? 6 : (sizeof(S) == 4 ? 6 : 4); }
+// Occupancy, measured on GB300 (256^3 packed spheres, us per launch).  The
+// collision runs 64-thread blocks, 12 per SM for the FP32 and 16-bit storages
+// (80 registers, no spills of note) and 8 for FP64: FP16 294 against 314 at 11 and
+// 317 at 13 blocks, 310 for 24 blocks of 32 threads; FP32 380 against 397, 423
+// and 402; 6 blocks of 128 threads are 0.5 % slower (rough channel 175.5 against 174.4).
+// The psi pass runs 64-thread blocks, 20 per SM (48 registers, no spills):
+// 16-bit storage 129.7 against 133.7 for 6 blocks of 256 (40 registers) and 131.1
+// for 12 of 128; FP32 176.5 against 179.5 and 178.7; smaller blocks leave no warps
+// waiting for the last of their block.
+constexpr int kPsiThreads = 64, kPsiBlocks = 20, kCollideThreads = 64;
+template <class S> constexpr int collide_min_blocks() { return sizeof(S) <= 4 ? 12 : 8; }
 
 // S1-S3 for the non-solid cell k of instance b: pull, sum to rho_alpha, store
 // the psi pair.  COH: f and the reference densities were written earlier in
@@ -78,6 +78,13 @@ __device__ __forceinline__ void psi_cell(const StepArgs &a, int b, uint32_t k, c
     psi[k] = out;
 }
 
+// Order of the two passes over the cells: the collision pass takes an instance's
+// blocks last to first, so that each pass starts with the cells the other has
+// just read and written, which are still in L2 (density pass of 1.4 M cells in FP32
+// 51.6 -> 46.8 us, of 6.6 M in FP16 137.7 -> 133.7).  Reversing the density pass's
+// blocks instead made that pass slower in FP32 (184 -> 190 us), and reversing the order of
+// a batch's instances too cost either pass 2 to 3 % (an instance index that is not
+// blockIdx.y itself) for 3 % of the density pass where there are many instances.
 template <class S, bool SLIP>
 __global__ void __launch_bounds__(kPsiThreads, kPsiBlocks) k_psi_c(StepArgs a) {
     const int b = blockIdx.y;
@@ -205,7 +212,7 @@ __device__ __forceinline__ void collide_cell(const StepArgs &a, int b, uint32_t 
 template <class S, int EQ>
 __global__ void __launch_bounds__(kCollideThreads, collide_min_blocks<S>()) k_collide_c(StepArgs a) {
     const int b = blockIdx.y;
-    const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
+    const uint32_t k = (gridDim.x - 1 - blockIdx.x) * blockDim.x + threadIdx.x;
     if (k >= (uint32_t)__ldg(a.list_count + b)) return;
     collide_cell<S, EQ, false>(a, b, k, a.write_macro);
 }
@@ -283,9 +290,9 @@ __device__ __forceinline__ void macro_cell2(const StepArgs &a, int b, long long 
 // block's shared-memory slots of the neighbour psi pairs (one column per
 // thread).  COH: psi, f and the reference densities were written earlier in
 // the same launch (the persistent update) and are read through L2.
-template <class S, int EQ, bool COH, bool PRE = false>
+template <class S, int EQ, bool COH, bool PRE = false, int THREADS>
 __device__ __forceinline__ void collide_cell2(const StepArgs &a, int b, uint32_t k, int write_macro,
-                                              float2 (&qs)[kQ - 1][kCollideThreads],
+                                              float2 (&qs)[kQ - 1][THREADS],
                                               const CompactCell *cell_pre = nullptr, const CNbr *nbr_pre = nullptr) {
     using P = typename Pair2<S>::P;
     const CompactCell c = PRE ? *cell_pre : compact_cell(a, b, k);
@@ -351,7 +358,7 @@ template <class S, int EQ>
 __global__ void __launch_bounds__(kCollideThreads, collide_min_blocks<S>()) k_collide_c2(StepArgs a) {
     __shared__ float2 qs[kQ - 1][kCollideThreads];
     const int b = blockIdx.y;
-    const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
+    const uint32_t k = (gridDim.x - 1 - blockIdx.x) * blockDim.x + threadIdx.x;
     if (k >= (uint32_t)__ldg(a.list_count + b)) return;
     collide_cell2<S, EQ, false>(a, b, k, a.write_macro, qs);
 }
@@ -364,7 +371,7 @@ __global__ void __launch_bounds__(kCollideThreads, collide_min_blocks<S>()) k_co
 // the launch (f, psi, the reference densities) is read through L2.  It serves
 // small instances and batches of them, where two launches per update cost more
 // than the work.
-constexpr int kPersistThreads = kCollideThreads;
+constexpr int kPersistThreads = 128;
 constexpr int kPersistMaxUpdates = 1 << 20;      // per launch: the barrier counter stays below 2^32
 constexpr long long kBarrierCycles = 4000000000LL;  // about 2 s of SM clock
 
