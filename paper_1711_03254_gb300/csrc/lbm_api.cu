@@ -422,6 +422,12 @@ StepArgs step_args(lbm_ctx *ctx, int write_macro) {
     return a;
 }
 
+// Room for the FP64 fields on their way to or from the host: the side of f that
+// does not hold the state, which is written before it is read again (5 x 8 bytes
+// per cell against 38 values of at least 2).  Allocating and freeing it in each
+// call took about 1.1 ms at 256^3.
+double *field_scratch(lbm_ctx *ctx) { return (double *)ctx->f[ctx->cur ^ 1]; }
+
 // After persistent launches: LBM_ERR_TIMEOUT if a grid-wide barrier gave up
 // (its blocks then left the launch early and the state is not an update).
 lbm_status check_barrier(lbm_ctx *ctx) {
@@ -732,8 +738,7 @@ lbm_status lbm_set_fields(lbm_ctx *ctx, const double *rho1, const double *rho2, 
     if (!ctx->has_geometry) return ctx->fail(LBM_ERR_STATE, "lbm_set_fields: call lbm_set_geometry first");
     LBM_CUDA(cudaSetDevice(ctx->dev), "cudaSetDevice");
     const size_t cells = ctx->cells();
-    double *d = (double *)ctx->dalloc(cells * 5 * sizeof(double));
-    if (!d) return ctx->fail(LBM_ERR_OOM, "lbm_set_fields: device allocation failed");
+    double *d = field_scratch(ctx);
     cudaError_t e = cudaMemcpyAsync(d, rho1, cells * 8, cudaMemcpyHostToDevice, ctx->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d + cells, rho2, cells * 8, cudaMemcpyHostToDevice, ctx->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d + 2 * cells, u, cells * 24, cudaMemcpyHostToDevice, ctx->stream);
@@ -756,7 +761,6 @@ lbm_status lbm_set_fields(lbm_ctx *ctx, const double *rho1, const double *rho2, 
         e = launch_init(a);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-    ctx->dfree(d);
     if (e != cudaSuccess) return ctx->cuda_fail(e, "lbm_set_fields");
     // the shifted storages first write the reference densities (k_init_ref)
     ctx->launches += (ctx->cfg.precision == LBM_FP32_F16S || ctx->cfg.precision == LBM_FP32_BF16S) ? 2 : 1;
@@ -895,15 +899,13 @@ lbm_status lbm_get_fields(lbm_ctx *ctx, double *rho1, double *rho2, double *u) {
     if (!ctx->has_fields) return ctx->fail(LBM_ERR_STATE, "lbm_get_fields: no fields yet");
     LBM_CUDA(cudaSetDevice(ctx->dev), "cudaSetDevice");
     const size_t cells = ctx->cells();
-    double *d = (double *)ctx->dalloc(cells * 5 * sizeof(double));
-    if (!d) return ctx->fail(LBM_ERR_OOM, "lbm_get_fields: device allocation failed");
+    double *d = field_scratch(ctx);
     cudaError_t e = launch_macro_to_f64(ctx->macro, ctx->fp64(), d, d + cells, d + 2 * cells, ctx->g,
                                         ctx->cfg.batch, ctx->stream);
     if (e == cudaSuccess && rho1) e = cudaMemcpyAsync(rho1, d, cells * 8, cudaMemcpyDeviceToHost, ctx->stream);
     if (e == cudaSuccess && rho2) e = cudaMemcpyAsync(rho2, d + cells, cells * 8, cudaMemcpyDeviceToHost, ctx->stream);
     if (e == cudaSuccess && u) e = cudaMemcpyAsync(u, d + 2 * cells, cells * 24, cudaMemcpyDeviceToHost, ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-    ctx->dfree(d);
     if (e != cudaSuccess) return ctx->cuda_fail(e, "lbm_get_fields");
     ctx->launches += 1;
     return check_barrier(ctx);
