@@ -34,16 +34,16 @@ extern "C" {
 /* y = act(conv(x, w) + bias); y is BF16 (y_f32 = 0) or FP32 (y_f32 = 1) with
  * row stride ldy; relu != 0 applies max(., 0); bias may be NULL.  Runs as an
  * implicit GEMM on the tcgen05 tensor cores (M = output positions, N = Co,
- * K = taps x Ci), accumulated in tensor memory.  Two kernels:
+ * K = taps x Ci), accumulated in tensor memory.  Kernels:
  *  - resident tiles (k = 3, W <= 254): a run of output lines of one plane is
  *    one tile; TMA loads its input one padded plane at a time and the 9 taps
- *    of the plane are shifted views of that tile.  For Co >= 64 or Ci = 16,
- *    where two accumulator buffers fit the tensor memory, one persistent
- *    block per SM strides over the tiles (the epilogue of a tile overlapping
- *    the next tile's MMAs); otherwise each block computes one tile.  The
- *    automatic choice gives small grids fewer lines per tile, or blocks that
- *    compute a part of the output channels.  All give the same bits;
- *  - gathered tiles (k = 1, and k = 3 where no resident plan fits): 128
+ *    of the plane are shifted views of that tile.  Each block computes one
+ *    tile, two or three blocks to an SM; on request one persistent block per
+ *    SM strides over the tiles instead.  The automatic choice gives small
+ *    grids fewer lines per tile, or blocks that compute a part of the output
+ *    channels.  All give the same bits;
+ *  - k = 1 with Ci <= 64 and Co <= 32: FP32 FMAs, one position per thread;
+ *  - gathered tiles (other k = 1, and k = 3 where no resident plan fits): 128
  *    positions per block, each tap's rows gathered with 16-byte copies.
  * Additional argument rules: Co <= 256, y 16-byte aligned, ldy a multiple of
  * 8 (BF16) or 4 (FP32).  Errors: 1 bad argument (also when the resident

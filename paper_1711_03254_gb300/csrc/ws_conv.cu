@@ -339,6 +339,70 @@ __global__ void __launch_bounds__(TTHREADS) k_conv_fwd_tc(const bf16 *__restrict
     }
 }
 
+// ------------------------------------------------------------------ forward, 1x1x1 of few channels
+// Y[p, co] = b[co] + sum_ci W[co, ci] X[p, ci] for k = 1, Ci <= 64 and Co <= 32 (the
+// U-Net's head): one position per thread, FP32 FMAs on pairs of output channels,
+// the weights as FP32 in shared memory (broadcast reads).  The call moves 64 + 64
+// bytes per position for 32 -> 16 channels and is bound by that; as tensor-core
+// tiles each block's start, gather and epilogue for one MMA took 28 us at 64^3
+// (cold caches) against 17 here.
+constexpr int kHeadThreads = 128, kHeadMaxCi = 64, kHeadMaxCo = 32;
+template <int CO, bool OUT_F32>
+__global__ void __launch_bounds__(kHeadThreads) k_conv1_fwd(const bf16 *__restrict__ X, int ldx,
+                                                           const bf16 *__restrict__ Wt,
+                                                           const float *__restrict__ bias, void *__restrict__ Y,
+                                                           int ldy, long long P, int Ci, int relu) {
+    __shared__ __align__(16) float w[kHeadMaxCi][CO];
+    for (int i = threadIdx.x; i < Ci * CO; i += kHeadThreads) {
+        const int co = i / Ci, ci = i - co * Ci;
+        w[ci][co] = __bfloat162float(Wt[i]);
+    }
+    __syncthreads();
+    const long long p = (long long)blockIdx.x * kHeadThreads + threadIdx.x;
+    if (p >= P) return;
+    float2 acc[CO / 2];
+#pragma unroll
+    for (int c = 0; c < CO / 2; ++c) acc[c] = make_float2(0.f, 0.f);
+    const uint4 *x4 = reinterpret_cast<const uint4 *>(X + p * ldx);
+    for (int c0 = 0; c0 < Ci; c0 += 16) {
+        __align__(16) bf16 x[16];
+        *reinterpret_cast<uint4 *>(x) = x4[c0 / 8];
+        *reinterpret_cast<uint4 *>(x + 8) = x4[c0 / 8 + 1];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            const float f = __bfloat162float(x[e]);
+            const float2 f2 = make_float2(f, f);
+#pragma unroll
+            for (int c = 0; c < CO / 2; c += 2) {
+                const float4 v = *reinterpret_cast<const float4 *>(&w[c0 + e][2 * c]);
+                acc[c] = __ffma2_rn(f2, make_float2(v.x, v.y), acc[c]);
+                acc[c + 1] = __ffma2_rn(f2, make_float2(v.z, v.w), acc[c + 1]);
+            }
+        }
+    }
+    float o[CO];
+#pragma unroll
+    for (int c = 0; c < CO; ++c) {
+        o[c] = (c & 1) ? acc[c / 2].y : acc[c / 2].x;
+        if (bias) o[c] += __ldg(bias + c);
+        if (relu) o[c] = fmaxf(o[c], 0.f);
+    }
+    if (OUT_F32) {
+        float4 *d = reinterpret_cast<float4 *>((float *)Y + p * ldy);
+#pragma unroll
+        for (int c = 0; c < CO / 4; ++c) d[c] = make_float4(o[4 * c], o[4 * c + 1], o[4 * c + 2], o[4 * c + 3]);
+    } else {
+        uint4 *d = reinterpret_cast<uint4 *>((bf16 *)Y + p * ldy);
+#pragma unroll
+        for (int c = 0; c < CO / 8; ++c) {
+            __align__(16) bf16 h[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) h[e] = __float2bfloat16_rn(o[8 * c + e]);
+            d[c] = *reinterpret_cast<const uint4 *>(h);
+        }
+    }
+}
+
 // ------------------------------------------------------------------ forward, resident tiles (3x3x3)
 // k_conv3_fwd_res: the same convolution for k = 3 with the input tile held in
 // shared memory instead of gathered per tap.  A block owns the outputs of
@@ -1426,12 +1490,13 @@ static int res_tiles(int lt, int pitch, int W) { return ((lt - 1) * pitch + W + 
 // accumulators fit the tensor memory (tiles x Co <= 512 columns) and whose
 // ring of at least two stages fits shared memory (a plan that leaves one block
 // per SM counts 15 % slower).  Then blocks per SM and stages as measured best
-// on the U-Net's layers (batch 4): for Co >= 64 one block per SM with up to 4
-// stages (32^3 64->64: 521 TFLOP/s against 418 with two blocks of 3 stages;
-// 160->64: 625 against 466), for narrower outputs two blocks per SM with 2
-// stages each (64^3 96->32: 628 against 572 with 3 stages; 32->32: 484
-// against 470), and ties broken toward fewer lines.  That choice is made for
-// lines of 32 columns or more, where it was measured; at 16^3 it left a
+// on the U-Net's layers (batch 4, us): two blocks per SM, with up to 4 stages for
+// Co >= 64 (32^3 160->64: 94 against 110 for one block of 4 stages and 114 for the
+// persistent kernel; 64->64: 45, 53 and 50) and 2 stages for narrower outputs; for Co <= 32
+// tiles of at most 128 tensor-memory columns and three blocks (64^3 32->32: 99
+// against 103 for two blocks of up to 256 columns; 16->32: 63 against 67; four blocks
+// of 96 columns: 102).  Ties are broken toward fewer lines.  That choice is made
+// for lines of 32 columns or more, where it was measured; at 16^3 it left a
 // nearly empty second wave (96->96: 164 against 243 TFLOP/s), so narrower lines
 // keep the search's stages and blocks per SM.  Returns false if none fits.
 static constexpr int kSmemPerSM = 233472, kSmemPerBlockMax = 232448, kSmemReserved = 1024;
@@ -1443,7 +1508,8 @@ static bool res_plan(int W, int H, int Co, ResPlan &best) {
     double best_eff = -1.0;
     for (int by = 1; by <= H && by <= 254; ++by) {
         const int nt = res_tiles(by, pitch, W);
-        if (nt * Co > 512) break;
+        // narrow outputs: at most 128 columns, so that three blocks share an SM
+        if (nt * Co > (tuned && Co <= 32 ? 128 : 512)) break;
         int cols = 32;
         while (cols < nt * Co) cols *= 2;
         int per_sm = 512 / cols;
@@ -1487,12 +1553,11 @@ static bool res_plan(int W, int H, int Co, ResPlan &best) {
             --best.per_sm;
         return true;
     }
-    // blocks per SM and stages of the chosen tiles: one block with up to 4
-    // stages for Co >= 64, else up to two blocks with 2 stages each (two
-    // stages fit one block per SM whenever the search above found a plan)
+    // blocks per SM and stages of the chosen tiles (two stages fit one block per
+    // SM whenever the search above found a plan)
     const int ns_max = Co >= 64 ? 4 : 2;
     best.stages = 0;
-    for (int per_sm = Co >= 64 ? 1 : std::min(512 / best.cols, 2); per_sm >= 1 && !best.stages; --per_sm) {
+    for (int per_sm = std::min(512 / best.cols, Co <= 32 ? 3 : 2); per_sm >= 1 && !best.stages; --per_sm) {
         long long budget = (long long)kSmemPerSM / per_sm - kSmemReserved;
         if (budget > kSmemPerBlockMax) budget = kSmemPerBlockMax;
         for (int ns = ns_max; ns >= 2; --ns) {
@@ -1552,16 +1617,11 @@ static bool pers_plan(const ResPlan &res, int Co, ResPlan &p, uint32_t &buf_cols
     return false;
 }
 
-// The persistent forward kernel where it measured faster (U-Net layers, batch
-// 4, us): Co >= 64 (32^3 64->64: 50.1 against 52.8, 32->64: 29.1 against 34.0) and
-// 16-channel inputs; one block per tile for narrower outputs of wider inputs
-// (64^3 96->32: 252 against 366, 32->32: 103 against 134).  The automatic choice
-// also runs one block per tile where there is at most one tile per SM and
-// nothing to overlap (16^3 224->96: 38.3 against 43.1, one sample of 32^3 64->64: 18.5
-// against 20.3).
-static bool want_persistent(int Ci, int Co) {
-    return g_fwd_algo == 4 || (g_fwd_algo != 3 && (Co >= 64 || Ci <= 16));
-}
+// The persistent forward kernel runs on request only: two or three blocks of one
+// tile each per SM measured as fast or faster on every layer of the U-Net (batch 4,
+// us: 32^3 64->64 45 against 50, 160->64 94 against 114, 16^3 224->96 38 against 43, 64^3
+// 16->32 63 against 85; 32->64 29.6 against 29.0).
+static bool want_persistent() { return g_fwd_algo == 4; }
 
 // Small grids (automatic choice): a plan that leaves SMs idle, or one block per
 // SM where two would share its tensor core, is replaced by one with fewer lines
@@ -1644,11 +1704,10 @@ static int conv3_fwd_res(const void *x, int ldx, const void *w, const float *bia
                          const Act &a, int Ci, int Co, int relu, cudaStream_t s, ResPlan pl) {
     ResPlan pp;
     uint32_t buf_cols = 0;
-    bool persistent = want_persistent(Ci, Co) && pers_plan(pl, Co, pp, buf_cols);
+    bool persistent = want_persistent() && pers_plan(pl, Co, pp, buf_cols);
     int nco = 1;
     if (g_fwd_algo == 0) {
         ResPlan sp;
-        persistent = persistent && (long long)a.N * a.D * pl.nyt > sm_count();
         if (small_grid_plan(a, Ci, Co, pl, persistent, sp, nco)) {
             pl = sp;
             persistent = false;
@@ -1936,6 +1995,14 @@ int ws_conv3d_fwd(const void *x, int ldx, const void *w, const float *bias, void
         if (res_plan(W, H, Co, pl)) return conv3_fwd_res(x, ldx, w, bias, y, ldy, y_f32, a, Ci, Co, relu, s, pl);
         if (g_fwd_algo >= 2) return 1;
     }
+    const long long head_blocks = (P + kHeadThreads - 1) / kHeadThreads;
+    if (k == 1 && g_fwd_algo != 1 && Ci <= kHeadMaxCi && Co <= kHeadMaxCo && head_blocks <= 0x7FFFFFFFLL) {
+        auto fn = Co == 16 ? (y_f32 ? k_conv1_fwd<16, true> : k_conv1_fwd<16, false>)
+                           : (y_f32 ? k_conv1_fwd<32, true> : k_conv1_fwd<32, false>);
+        fn<<<(unsigned)head_blocks, kHeadThreads, 0, s>>>((const bf16 *)x, ldx, (const bf16 *)w, bias, y, ldy, P, Ci,
+                                                          relu);
+        return cudaGetLastError() == cudaSuccess ? 0 : 2;
+    }
     const int cols = Co <= 32 ? 32 : (Co <= 64 ? 64 : (Co <= 128 ? 128 : 256));
     const size_t smem = 2 * (size_t)TKC * (TBM * 32 + (size_t)Co * 32) + 2 * sizeof(uint64_t) + 16;
     static bool attr[2] = {false, false};
@@ -1976,10 +2043,9 @@ int ws_conv3d_plan(int which, int N, int D, int H, int W, int Ci, int Co, long l
         uint32_t buf_cols = 0;
         if (g_fwd_algo == 1 || !res_plan(W, H, Co, pl)) return -1;
         const long long tiles = (long long)N * D * pl.nyt;
-        bool pers = want_persistent(Ci, Co) && pers_plan(pl, Co, pp, buf_cols);
+        bool pers = want_persistent() && pers_plan(pl, Co, pp, buf_cols);
         ResPlan sp;
         int nco = 1;
-        if (g_fwd_algo == 0) pers = pers && tiles > sm_count();
         if (g_fwd_algo == 0 && small_grid_plan(a, Ci, Co, pl, pers, sp, nco)) {
             pl = sp;
             pers = false;

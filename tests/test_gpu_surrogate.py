@@ -255,3 +255,26 @@ def test_small_grids_keep_the_bits(env, shape, Ci, Co):
     assert ws.ws_tc_status() == 0
     for p, q in zip(*out):
         assert torch.equal(p, q)
+
+
+@pytest.mark.parametrize("P,Ci,Co", [(1, 16, 16), (127, 32, 16), (129, 48, 32), (1000, 64, 32), (256, 80, 16), (130, 32, 48)])
+@pytest.mark.parametrize("f32", [True, False])
+def test_pointwise_convolution(env, P, Ci, Co, f32):
+    """1x1x1 convolutions on both sides of the limits of the few-channel kernel
+    (Ci <= 64, Co <= 32), from and into channel slices, against FP64."""
+    torch, ws, _ = env
+    g = torch.Generator(device="cuda").manual_seed(P + Ci)
+    x = torch.randn((1, 1, 1, P, Ci + 8), generator=g, device="cuda").to(torch.bfloat16)[..., 8:]
+    w = (torch.randn((Co, 1, 1, 1, Ci), generator=g, device="cuda") * 0.2).to(torch.bfloat16)
+    b = torch.randn(Co, generator=g, device="cuda")
+    y = torch.full((1, 1, 1, P, Co + 8), 5.0, dtype=torch.float32 if f32 else torch.bfloat16, device="cuda")
+    ref = x.double().reshape(P, Ci) @ w.double().reshape(Co, Ci).T
+    for bias, relu in ((b, True), (None, False)):
+        ws.ws_conv3d_fwd(x, w, bias, y[..., :Co], relu)
+        want = ref + (bias.double() if bias is not None else 0.0)
+        want = want.clamp(min=0.0) if relu else want
+        # FP32 sums of at most 80 products; a BF16 result adds half a unit of 2^-8
+        tol = 1e-5 if f32 else 2.0 ** -8
+        got = y[..., :Co].double().reshape(P, Co)
+        assert float((got - want).abs().max()) <= tol * float(want.abs().max())
+        assert bool((y[..., Co:] == 5.0).all())
