@@ -416,7 +416,10 @@ def main():
     strategy = lbm.lbm_resolved_kernel(sim.ctx, args.steps)
     kernel_name = {"psi": "k_psi", "collide": "k_collide", "fused": "k_fused", "cluster": "k_cluster"}[part]
     if strategy == "persistent":
-        kernel_name = "k_persist_c"
+        # on chip where the storage computes in FP32 and an instance has at most
+        # 8192 non-solid cells (and no wall slip, which no workload here has)
+        onchip = args.precision != "fp64" and int((t != 1).sum(axis=(1, 2, 3)).max()) <= 8192
+        kernel_name = "k_onchip_c" if onchip else "k_persist_c"
     if strategy == "compact":
         # compact layout: packed-pair update for the FP32-arithmetic storages
         kernel_name += {"psi": "_c", "collide": "_c" if args.precision == "fp64" else "_c2"}[part]

@@ -101,7 +101,7 @@ int ws_conv3d_bwd_weight_algo(int algo);
  * allocation).  which = 0: forward (also the data gradient with Ci and Co
  * exchanged); out[0..13] = persistent kernel (0/1), lines per tile, tiles per
  * plane, line pitch (W + 2), 128-row M tiles per tile, stages, tensor-memory
- * columns, blocks per SM, bytes of one K half of a stage's input, stage bytes,
+ * columns, blocks per SM, half the bytes of a stage's input tile, stage bytes,
  * TMA bytes per stage, dynamic shared memory requested, blocks in the grid,
  * columns per accumulator buffer (persistent kernel, else 0).  which = 1:
  * weight gradient; out[0..15] = dz-slot kernel (0: none, 1: without, 2: with

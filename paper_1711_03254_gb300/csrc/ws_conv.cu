@@ -14,11 +14,14 @@
 //   k_conv3_fwd_res, k_conv3_fwd_pers   forward (and data gradient) for 3x3x3, the
 //                                       input tile resident in shared memory (TMA),
 //                                       the taps as shifted descriptors; one block
-//                                       per tile or one persistent block per SM
+//                                       per tile or (on request) one persistent
+//                                       block per SM
 //   k_conv3_wgrad_res, k_conv3_wgrad_dz weight gradient for 3x3x3 from TMA line boxes,
-//                                       tap pairs or dz slots as M rows
+//                                       tap pairs or dz slots as M rows, the latter
+//                                       with copies of dY as N columns
 //   k_conv_fwd_tc, k_conv_wgrad_tc      the gathered kernels (cp.async, two stages):
 //                                       1x1x1 and the shapes no resident plan fits
+//   k_conv1_fwd                         1x1x1 of few channels (FP32 FMAs)
 // The host picks among them (ws_conv3d_fwd_algo, ws_conv3d_bwd_weight_algo).
 //
 // Activations are channels-last with a row stride (ld) and a channel offset,
@@ -408,18 +411,20 @@ __global__ void __launch_bounds__(kHeadThreads) k_conv1_fwd(const bf16 *__restri
 // shared memory instead of gathered per tap.  A block owns the outputs of
 // `by` consecutive lines of one plane.  Its input is loaded plane by plane by
 // TMA: for the K-step (16-channel chunk c, plane offset dz) one box of
-// (by + 2) lines x (W + 2) columns x 8 channels per K half, halo included
-// (outside the volume the tensor map fills zeros), lands as rows of 16 bytes
-// in the order (line, column).  In that layout an output row q = l (W + 2) + x
+// (by + 2) lines x (W + 2) columns x 16 channels, halo included (outside the
+// volume the tensor map fills zeros), lands as rows of 32 bytes in the order
+// (line, column).  In that layout an output row q = l (W + 2) + x
 // and its input at tap (dy, dx) are a fixed distance apart, dy (W + 2) + dx
 // rows, so the A operand of a tap is the same shared-memory tile seen through
-// a descriptor that starts 16 (dy (W + 2) + dx) bytes further: the 9 taps of a
+// a descriptor that starts 32 (dy (W + 2) + dx) bytes further: the 9 taps of a
 // plane cost one load.  The rows between two lines (the x halo) are computed
-// and discarded.  The no-swizzle K-major layout has rows 16 bytes apart
-// within a core matrix and, with a stride byte offset of 128, across core
-// matrices, so any 16-byte start is a valid tile; the two K halves of a chunk
-// are separate boxes one leading byte offset apart.  The weights of the 9 taps
-// of (c, dz) arrive by TMA as [tap][K half][Co rows] tiles.
+// and discarded.  Tiles use the 32-byte swizzle, which depends on the address
+// alone, so a tile may start at any row of what TMA wrote.  The weights of the
+// 9 taps of (c, dz) arrive by one TMA load as [tap][Co rows].  Rows of 16
+// bytes without swizzle (two loads and 18) moved twice the TMA rows: 64^3
+// 32->32, batch 4, 441 TFLOP/s against 539.  What bounds it now is the MMA: with the
+// loads left out after the first stages 64^3 32->32 took 106 of its 107 us, some 64
+// clocks per M128 N32 K16 MMA with two blocks per SM, (A + B bytes) / 64 + 20.
 //
 // With nco > 1 a block computes Co of the nco x Co output channels (small grids,
 // see small_grid_plan).
@@ -963,15 +968,16 @@ __global__ void __launch_bounds__(WTTHREADS) k_conv_wgrad_tc(const bf16 *__restr
 // k_conv3_wgrad_res: dW[co][t][ci] = sum_p dY[p][co] X[p + t - 1][ci] with the
 // positions of a run of `by` lines as K, M = 128 rows of (tap pair (dz, dy),
 // ci) and N = Co.  Per K-block (by lines y0.. of plane z of sample n) TMA
-// loads, for each (dz, dy) of the block's tile and each 8-channel group, the
-// box of X at lines y0 + dy - 1 .., plane z + dz - 1, columns -1 .. W (one
-// region of 16-byte rows in the order (line, column)), and the box of dY at
+// loads, for each (dz, dy) of the block's tile and each 16-channel group, the
+// box of X at lines y0 + dy - 1 .., plane z + dz - 1, columns -1 .. W (32-byte
+// rows in the order (line, column), in the 32-byte swizzle; a group takes two
+// regions), and the box of dY at
 // lines y0 .., columns 0 .. W + 1 (zeros beyond W, so the two columns that
 // pad each line add nothing).  In that order the input of tap dx for the
 // position in row q sits in row q + dx of the X region: the three dx taps are
-// the same regions seen through descriptors 16 dx bytes apart.  Both operands
-// are MN-major (8 channels of one position form a 16-byte row; K pairs 128 B
-// apart, 8-channel groups one region apart).  M holds 128 / ci_blk tap pairs
+// the same groups seen through descriptors 32 dx bytes apart.  Both operands
+// are MN-major (16 channels of one position form a 32-byte row, 8 positions
+// 256 B, 16-channel groups two regions apart).  M holds 128 / ci_blk tap pairs
 // of ci_blk channels; a block owns one such tile of one channel block and a
 // range of K-blocks, accumulates [dx][M][Co] in tensor memory and writes its
 // partial rows part[pb][t * Ci + ci][co]; k_wgrad_sum adds the partials in
