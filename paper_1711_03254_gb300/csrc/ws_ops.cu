@@ -20,19 +20,28 @@ using bf16 = __nv_bfloat16;
 // than the element.  One thread per element with 64-bit divisions took, at 64^3
 // positions: ReLU adjoint of 4 x 32 channels 103 us, upsampling to 64 channels
 // 108, pooling of 32 channels 15.2, the cast of 16 channels 14.2.
-template <int V> struct Vec;
-template <> struct Vec<1> {
-    bf16 v[1];
-    __device__ __forceinline__ void load(const bf16 *p) { v[0] = *p; }
-    __device__ __forceinline__ void store(bf16 *p) const { *p = v[0]; }
-};
-template <> struct Vec<8> {
-    bf16 v[8];
-    __device__ __forceinline__ void load(const bf16 *p) {
-        *reinterpret_cast<uint4 *>(v) = *reinterpret_cast<const uint4 *>(p);
+template <int V, class T = bf16> struct Vec {
+    // aligned for the 16-byte accesses below, wherever the compiler keeps it
+    alignas(V * sizeof(T) % 16 == 0 ? 16 : alignof(T)) T v[V];
+    __device__ __forceinline__ void load(const T *p) {
+        if constexpr (V * sizeof(T) % 16 == 0) {
+#pragma unroll
+            for (int j = 0; j < (int)(V * sizeof(T) / 16); ++j)
+                reinterpret_cast<uint4 *>(v)[j] = reinterpret_cast<const uint4 *>(p)[j];
+        } else {
+#pragma unroll
+            for (int j = 0; j < V; ++j) v[j] = p[j];
+        }
     }
-    __device__ __forceinline__ void store(bf16 *p) const {
-        *reinterpret_cast<uint4 *>(p) = *reinterpret_cast<const uint4 *>(v);
+    __device__ __forceinline__ void store(T *p) const {
+        if constexpr (V * sizeof(T) % 16 == 0) {
+#pragma unroll
+            for (int j = 0; j < (int)(V * sizeof(T) / 16); ++j)
+                reinterpret_cast<uint4 *>(p)[j] = reinterpret_cast<const uint4 *>(v)[j];
+        } else {
+#pragma unroll
+            for (int j = 0; j < V; ++j) p[j] = v[j];
+        }
     }
 };
 
@@ -207,17 +216,11 @@ __global__ void k_to_bf16(const float *__restrict__ x, int ldx, bf16 *__restrict
     if (i >= total) return;
     const I cv = (I)(C / V), p = i / cv;
     const int c = (int)(i - p * cv) * V;
-    const float *s = x + (long long)p * ldx + c;
-    float f[V];
-    if constexpr (V == 8) {
-        *reinterpret_cast<float4 *>(f) = *reinterpret_cast<const float4 *>(s);
-        *reinterpret_cast<float4 *>(f + 4) = *reinterpret_cast<const float4 *>(s + 4);
-    } else {
-        f[0] = s[0];
-    }
+    Vec<V, float> f;
+    f.load(x + (long long)p * ldx + c);
     Vec<V> o;
 #pragma unroll
-    for (int e = 0; e < V; ++e) o.v[e] = __float2bfloat16_rn(f[e]);
+    for (int e = 0; e < V; ++e) o.v[e] = __float2bfloat16_rn(f.v[e]);
     o.store(y + (long long)p * ldy + c);
 }
 
