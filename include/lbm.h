@@ -79,9 +79,10 @@ typedef enum {
 typedef enum {
     LBM_KERNEL_AUTO = 0,     /* compact when the grid fits its coordinate limits, else two-pass;
                                 for n >= 8 updates the persistent update of instances that fit
-                                a cluster's shared memory (any number of them), or of at most
-                                65,536 non-solid cells in all (32,768 inside
-                                lbm_run_to_steady's graphs); no wall slip */
+                                a cluster's shared memory (many of more than 5,120 cells, which
+                                leave SMs idle there, take the compact one) or of at most 65,536
+                                non-solid cells in all (32,768 inside lbm_run_to_steady's
+                                graphs); no wall slip */
     LBM_KERNEL_TWO_PASS = 1, /* density pre-pass, then stream+collide, over the non-solid cells */
     LBM_KERNEL_FUSED = 2,    /* single read of f: z-marching tiles with a recomputed density halo */
     LBM_KERNEL_CLUSTER = 3,  /* persistent: one thread-block cluster per instance, n updates per launch */

@@ -67,7 +67,7 @@ struct lbm_ctx {
     bool persist_used = false; // a persistent launch ran since the flag was last read
     long long bar_cycles = 4000000000LL;  // bound on a barrier wait (about 2 s of SM clock)
     unsigned bar_missing = 0;  // failure test: arrivals the barriers wait for that never come
-    int onchip = 0;  // threads per block of the on-chip persistent update (0: does not fit)
+    OnchipPlan onchip;  // on-chip persistent update of this geometry (threads 0: does not fit)
     FcPlan fplan{};  // single-read fused update on the compact layout (ok when it fits)
     std::vector<uint32_t> plane_start;  // compact index of each plane's first cell (instance 0), nz + 1
     bool half_step = false;             // the density pass of a split update has run
@@ -222,6 +222,37 @@ const char *check_params(const lbm_instance_params *per_instance, int batch) {
     return nullptr;
 }
 
+// Whether n updates of instances kept in a thread-block cluster's shared memory
+// take less time than n pairs of launches: us per update, from measurements on
+// GB300.  The clusters run in waves of those that are resident together.  An
+// update of a wave takes 2.6 to 3.3 us (barriers, issue) and more by the share of
+// pulls that leave the block, which follows from how far apart the z and y
+// neighbours lie in the cell order (16 x 16^3 3.5, 20^3 4.9, a channel of 4 x 4
+// cells across 3.2); loading and storing the state takes 5.3 us a wave.  Two
+// launches take 5 us in the steady loop's graphs and 7.5 stepped, plus 66 ps per
+// cell of the blocks' 64, FP32 88 ps where f no longer stays in L2.
+// One wave always pays: 16^3 3.1 against 12.3 us, 16 channels of 4 x 128 x 4 3.6
+// against 12.3.  So do more waves of clusters of up to 8 blocks, mostly: 104 slugs
+// of 3840 cells 22.5 against 37.0, 256 x 16^3 62.7 against 100 (FP32), 63 against 80
+// (FP16).  A GPC holds one cluster of 11 to 16 blocks, so there fewer cells are
+// resident: 104 x 18^3 57.6 against 63.6 in FP32 but 54.5 against 47.2 in FP16;
+// 256 x 19^3 170 against 158 and 162 against 127; 104 x 5184 cells in FP16 at n = 8
+// 61.3 against 41.6.
+bool onchip_pays(const lbm_ctx *ctx, int n) {
+    if (ctx->onchip.waves <= 1) return true;
+    const double kmax = (double)ctx->list_max, block = ctx->onchip.threads;
+    const double plane = ctx->g.nz > 1 ? kmax / ctx->g.nz : 0.0, row = kmax / ((double)ctx->g.nz * ctx->g.ny);
+    // of the 19 directions 10 have a z component, 6 of the others a y component
+    const double away = (10.0 * std::min(1.0, plane / block) + 6.0 * std::min(1.0, row / block)) / 19.0;
+    // (full equilibrium: 5 % more, third-order regularisation 8 %)
+    const double more = 1.0 + (ctx->cfg.eq_order == 1 ? 0.05 : 0.0) + (ctx->cfg.reg_order == 3 ? 0.08 : 0.0);
+    const double wave = more * (2.6 + 0.7 * std::min(1.0, kmax / 4096.0) + 450e-6 * away * kmax) + 5.3 / n;
+    const double cells = (double)ctx->cfg.batch * 64.0 * std::ceil(kmax / 64.0);
+    double two = (ctx->in_graph ? 5.0 : 7.5) + 66e-6 * cells;
+    if (ctx->cfg.precision == LBM_FP32) two += 22e-6 * std::max(0.0, cells - 200e3);
+    return (double)ctx->onchip.waves * wave < two;
+}
+
 // Strategy for an n-update call.  AUTO: the compact two-pass update when the
 // grid fits its packed coordinates, the dense two-pass one otherwise.
 lbm_kernel resolve_kernel(const lbm_ctx *ctx, int n) {
@@ -229,15 +260,9 @@ lbm_kernel resolve_kernel(const lbm_ctx *ctx, int n) {
     // memory; where they do not, its layout's two-pass update runs
     if (ctx->kernel == LBM_KERNEL_FUSED_COMPACT) return ctx->fplan.ok ? LBM_KERNEL_FUSED_COMPACT : LBM_KERNEL_COMPACT;
     if (ctx->kernel != LBM_KERNEL_AUTO) return ctx->kernel;
-    // instances that fit a thread-block cluster's shared memory stay there for
-    // all n updates, however many instances there are (GB300, FP32, us per
-    // update against two launches each: 16^3 3.1 against 12.3, 16 channels of
-    // 4 x 128 x 4 3.6 against 12.3, 104 slugs of 3840 cells 22.5 against 37.0,
-    // 256 x 16^3 62.7 against 100; in the steady loop's CUDA graphs 4.3 against
-    // 8.6, 4.9 against 9.5, 24.5 against 35.8, 65.9 against 98.4)
-    if (ctx->onchip > 0 && !ctx->slip_on() && n >= 8) return LBM_KERNEL_PERSISTENT;
-    // other small problems: one cooperative launch for the n updates, each thread
-    // keeping its cell, beats two launches per update (GB300, FP32, us per
+    if (ctx->onchip.threads > 0 && !ctx->slip_on() && n >= 8 && onchip_pays(ctx, n)) return LBM_KERNEL_PERSISTENT;
+    // other small problems (on chip too where the instances fit, in a few waves of
+    // clusters): one cooperative launch for the n updates, each thread keeping its cell, beats two launches per update (GB300, FP32, us per
     // update, stepped from the host: 24^3 5.9 against 12.3, 32^3 6.7 against
     // 12.3; in the steady loop's CUDA graphs, where launches are cheap: 24^3 7.1
     // against 8.7, 32^3 8.0 against 9.4; FP64, stepped: 16^3 28.1 against 34.8,
@@ -363,7 +388,7 @@ lbm_status build_cell_lists(lbm_ctx *ctx) {
     ctx->dfree(rowcnt);
     if (e != cudaSuccess) return ctx->cuda_fail(e, "cell lists");
     ctx->launches += ctx->compact_ok ? 5 : 4;
-    ctx->onchip = ctx->compact_ok ? onchip_threads(step_args(ctx, 0)) : 0;
+    ctx->onchip = ctx->compact_ok ? onchip_plan(step_args(ctx, 0)) : OnchipPlan{};
     return plan_fused_compact(ctx);
 }
 
@@ -418,7 +443,7 @@ StepArgs step_args(lbm_ctx *ctx, int write_macro) {
     a.bar_cycles = ctx->bar_cycles;
     a.bar_missing = ctx->bar_missing;
     // (the failure test of the grid-wide barriers runs the kernel that has them)
-    a.onchip = !a.slip && a.bar_missing == 0 ? ctx->onchip : 0;
+    a.onchip = !a.slip && a.bar_missing == 0 ? ctx->onchip.threads : 0;
     return a;
 }
 

@@ -32,9 +32,9 @@ extern template cudaError_t launch_persist_t<double>(const StepArgs &, int);
 extern template cudaError_t launch_persist_t<float>(const StepArgs &, int);
 extern template cudaError_t launch_persist_t<__half>(const StepArgs &, int);
 extern template cudaError_t launch_persist_t<__nv_bfloat16>(const StepArgs &, int);
-extern template int onchip_threads_t<float>(const StepArgs &);
-extern template int onchip_threads_t<__half>(const StepArgs &);
-extern template int onchip_threads_t<__nv_bfloat16>(const StepArgs &);
+extern template OnchipPlan onchip_plan_t<float>(const StepArgs &);
+extern template OnchipPlan onchip_plan_t<__half>(const StepArgs &);
+extern template OnchipPlan onchip_plan_t<__nv_bfloat16>(const StepArgs &);
 extern template cudaError_t launch_onchip_t<float>(const StepArgs &, int);
 extern template cudaError_t launch_onchip_t<__half>(const StepArgs &, int);
 extern template cudaError_t launch_onchip_t<__nv_bfloat16>(const StepArgs &, int);
@@ -87,12 +87,12 @@ cudaError_t launch_compact(const StepArgs &a, int parts) {
     return cudaErrorInvalidValue;
 }
 
-int onchip_threads(const StepArgs &a) {
+OnchipPlan onchip_plan(const StepArgs &a) {
     switch (a.precision) {
-    case LBM_FP32: return onchip_threads_t<float>(a);
-    case LBM_FP32_F16S: return onchip_threads_t<__half>(a);
-    case LBM_FP32_BF16S: return onchip_threads_t<__nv_bfloat16>(a);
-    default: return 0;
+    case LBM_FP32: return onchip_plan_t<float>(a);
+    case LBM_FP32_F16S: return onchip_plan_t<__half>(a);
+    case LBM_FP32_BF16S: return onchip_plan_t<__nv_bfloat16>(a);
+    default: return {};
     }
 }
 

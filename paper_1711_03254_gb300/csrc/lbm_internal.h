@@ -105,8 +105,13 @@ int fused_tile_count();
 // nsteps updates in one persistent launch, one thread-block cluster per instance
 cudaError_t launch_cluster(const StepArgs &a, int nsteps);
 cudaError_t launch_persist(const StepArgs &a, int nsteps);
-// threads per block of the on-chip persistent update (lbm_onchip.cuh); 0 where it does not apply
-int onchip_threads(const StepArgs &a);
+// the on-chip persistent update (lbm_onchip.cuh): threads per block (0 where it does not
+// apply) and waves of resident clusters that all instances take
+struct OnchipPlan {
+    int threads = 0;
+    long long waves = 0;
+};
+OnchipPlan onchip_plan(const StepArgs &a);
 int cluster_size_for(long long n);
 cudaError_t launch_init(const InitArgs &a);
 cudaError_t launch_links(const uint8_t *type, uint32_t *link, const Grid &g, int batch, cudaStream_t s);

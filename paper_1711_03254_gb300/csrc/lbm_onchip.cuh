@@ -186,19 +186,19 @@ template <class S, int EQ> cudaError_t onchip_config(const StepArgs &a, int thre
                                 (int)onchip_smem<S>(kOnchipMaxThreads));
 }
 
-// Threads per block (a power of two from 64 to 512, a cluster of at most 16
-// blocks holding an instance); 0 where the on-chip update does not apply.  The
+// Plan: threads per block (a power of two from 64 to 512, a cluster of at most 16
+// blocks holding an instance) and waves of clusters; 0 threads where the on-chip
+// update does not apply.  The
 // fewest threads with which all instances run at once, because cells spread
 // over more SMs wait less for each other's instructions (one 16^3: 3.06 us per
 // update at 256 threads, 3.48 at 512); where they do not all fit, what needs
 // the fewest waves of clusters, and of those the most threads (104 slugs of
 // 3840 cells: 22.5 us at 512 threads, 24.7 at 256; 256 x 16^3: 62.7 and 74.3).
-template <class S> int onchip_threads_t(const StepArgs &a) {
-    int best = 0;
-    if (a.slip || a.kmax < 1) return 0;
+template <class S> OnchipPlan onchip_plan_t(const StepArgs &a) {
+    OnchipPlan best;
+    if (a.slip || a.kmax < 1) return best;
     dispatch_variant(collide_variant(a) & 3, [&](auto v) {
         constexpr int EQ = decltype(v)::value & 3;
-        long long best_waves = 0;
         for (int c = 64; c <= kOnchipMaxThreads; c *= 2) {
             if ((long long)a.kmax > (long long)c * kOnchipMaxCluster) continue;
             cudaLaunchConfig_t cfg;
@@ -210,9 +210,9 @@ template <class S> int onchip_threads_t(const StepArgs &a) {
                 continue;
             }
             const long long waves = ((long long)a.batch + n - 1) / n;
-            if (best == 0 || waves < best_waves || (waves == best_waves && waves > 1)) {
-                best = c;
-                best_waves = waves;
+            if (best.threads == 0 || waves < best.waves || (waves == best.waves && waves > 1)) {
+                best.threads = c;
+                best.waves = waves;
             }
         }
     });

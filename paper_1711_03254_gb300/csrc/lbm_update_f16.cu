@@ -8,7 +8,7 @@ namespace lbm {
 template cudaError_t launch_two_pass_t<__half>(const StepArgs &);
 template cudaError_t launch_compact_t<__half>(const StepArgs &, int);
 template cudaError_t launch_persist_t<__half>(const StepArgs &, int);
-template int onchip_threads_t<__half>(const StepArgs &);
+template OnchipPlan onchip_plan_t<__half>(const StepArgs &);
 template cudaError_t launch_onchip_t<__half>(const StepArgs &, int);
 
 }  // namespace lbm

@@ -8,7 +8,7 @@ namespace lbm {
 template cudaError_t launch_two_pass_t<float>(const StepArgs &);
 template cudaError_t launch_compact_t<float>(const StepArgs &, int);
 template cudaError_t launch_persist_t<float>(const StepArgs &, int);
-template int onchip_threads_t<float>(const StepArgs &);
+template OnchipPlan onchip_plan_t<float>(const StepArgs &);
 template cudaError_t launch_onchip_t<float>(const StepArgs &, int);
 
 }  // namespace lbm
