@@ -83,6 +83,10 @@ def alg_bytes_per_cell(part: str, precision: str) -> int:
     if part == "persistent":
         # each update of the persistent launch: both passes of the compact update
         return alg_bytes_per_cell("psi", precision) + alg_bytes_per_cell("collide", precision)
+    if part == "onchip":
+        # the whole launch, whatever its number of updates: f and the reference pairs in
+        # and out, packed coordinates and geometry word in, the last update's five fields out
+        return 76 * s + 4 + 4 + 2 * ref + 5 * t
     return 76 * s + 4 + 2 * ref  # fused, and each update of a cluster launch
 # DRAM traffic of the dominant kernel from one ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum of a launch / its fluid cells),
@@ -415,10 +419,8 @@ def main():
     part_ms, part_launches = timing[part]
     strategy = lbm.lbm_resolved_kernel(sim.ctx, args.steps)
     kernel_name = {"psi": "k_psi", "collide": "k_collide", "fused": "k_fused", "cluster": "k_cluster"}[part]
+    onchip = lbm.lbm_resolved_onchip(sim.ctx, args.steps)
     if strategy == "persistent":
-        # on chip where the storage computes in FP32 and an instance has at most
-        # 8192 non-solid cells (and no wall slip, which no workload here has)
-        onchip = args.precision != "fp64" and int((t != 1).sum(axis=(1, 2, 3)).max()) <= 8192
         kernel_name = "k_onchip_c" if onchip else "k_persist_c"
     if strategy == "compact":
         # compact layout: packed-pair update for the FP32-arithmetic storages
@@ -432,6 +434,8 @@ def main():
     impl_bytes = alg_bytes_per_cell("fused_compact" if strategy == "fused_compact" else
                                     ("persistent" if strategy == "persistent" else part), args.precision)
     updates_per_launch = args.steps if part == "cluster" else 1
+    if onchip:
+        impl_bytes = round(alg_bytes_per_cell("onchip", args.precision) / updates_per_launch, 3)
     avg_s = part_ms / part_launches / 1e3
     achieved = method_bytes * fluid * updates_per_launch / avg_s / 1e9
     key = f"{kernel_name}/{args.precision}/{args.workload}"
@@ -460,6 +464,10 @@ def main():
             roof["step_traffic_bytes_per_fluid_cell"] = step_tr
             roof["wasted_traffic_ratio"] = round(step_tr / method_bytes, 3)
 
+    if onchip:
+        # the state stays in shared memory: an update waits for barriers and remote loads,
+        # and f's bytes (the figures above) do not cross DRAM in each
+        roof["bound"] = "latency"
     fl = FP64_FLOPS.get(kernel_name)
     if args.precision == "fp64" and fl and fl["src"] == sources_hash(fl["files"]):
         # FP64 arithmetic: the FP64 pipe, not HBM, bounds the update

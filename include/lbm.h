@@ -294,6 +294,10 @@ lbm_status lbm_set_kernel(lbm_ctx *ctx, lbm_kernel kernel);
  * the geometry, so call it after lbm_set_geometry).  Returns -1 for a NULL
  * context. */
 int lbm_resolved_kernel(const lbm_ctx *ctx, int n);
+/* 1 if lbm_step(ctx, n) would run LBM_KERNEL_PERSISTENT with every instance in a
+ * thread-block cluster's shared memory (f read and written once per call, not once
+ * per update), else 0.  Depends on the geometry. */
+int lbm_resolved_onchip(const lbm_ctx *ctx, int n);
 
 /* Tiling of the fused kernel: tile 0 = 32x8, 1 = 32x4, 2 = 64x4, 3 = 32x16
  * cells per thread block, each marching zchunk planes; -1 selects the

@@ -222,6 +222,10 @@ const char *check_params(const lbm_instance_params *per_instance, int batch) {
     return nullptr;
 }
 
+// Whether LBM_KERNEL_PERSISTENT keeps the instances on chip (the failure test of the
+// grid-wide barriers runs the kernel that has them).
+bool runs_onchip(const lbm_ctx *ctx) { return ctx->onchip.threads > 0 && !ctx->slip_on() && ctx->bar_missing == 0; }
+
 // Whether n updates of instances kept in a thread-block cluster's shared memory
 // take less time than n pairs of launches: us per update, from measurements on
 // GB300.  The clusters run in waves of those that are resident together.  An
@@ -442,8 +446,7 @@ StepArgs step_args(lbm_ctx *ctx, int write_macro) {
     a.bar = ctx->bar;
     a.bar_cycles = ctx->bar_cycles;
     a.bar_missing = ctx->bar_missing;
-    // (the failure test of the grid-wide barriers runs the kernel that has them)
-    a.onchip = !a.slip && a.bar_missing == 0 ? ctx->onchip.threads : 0;
+    a.onchip = runs_onchip(ctx) ? ctx->onchip.threads : 0;
     return a;
 }
 
@@ -648,6 +651,10 @@ lbm_status lbm_set_kernel(lbm_ctx *ctx, lbm_kernel kernel) {
 long long lbm_launch_count(const lbm_ctx *ctx) { return ctx ? ctx->launches : 0; }
 
 int lbm_resolved_kernel(const lbm_ctx *ctx, int n) { return ctx ? (int)resolve_kernel(ctx, n) : -1; }
+
+int lbm_resolved_onchip(const lbm_ctx *ctx, int n) {
+    return ctx && resolve_kernel(ctx, n) == LBM_KERNEL_PERSISTENT && runs_onchip(ctx) ? 1 : 0;
+}
 
 lbm_status lbm_timing_begin(lbm_ctx *ctx, int max_launches) {
     if (!ctx) return LBM_ERR_ARG;
@@ -1362,7 +1369,7 @@ lbm_status lbm_run_to_steady(lbm_ctx *ctx, int check_every, double tol, int max_
     if (hres) cudaFreeHost(hres);
     cudaStreamDestroy(cs);
     if (e != cudaSuccess) return ctx->cuda_fail(e, "lbm_run_to_steady");
-    if (kres == LBM_KERNEL_PERSISTENT && !step_args(ctx, 0).onchip) {
+    if (kres == LBM_KERNEL_PERSISTENT && !runs_onchip(ctx)) {
         ctx->persist_used = true;
         const lbm_status bs = check_barrier(ctx);
         if (bs != LBM_OK) return bs;

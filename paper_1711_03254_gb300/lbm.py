@@ -244,6 +244,14 @@ def lbm_resolved_kernel(ctx, n: int = 2) -> str:
     return {v: name for name, v in KERNELS.items()}.get(k, str(k))
 
 
+def lbm_resolved_onchip(ctx, n: int = 2) -> bool:
+    """Whether lbm_step(ctx, n) would keep every instance in a thread-block
+    cluster's shared memory for the n updates."""
+    L = library()
+    L.lbm_resolved_onchip.argtypes = [ctypes.c_void_p, ctypes.c_int]
+    return bool(L.lbm_resolved_onchip(ctx, int(n)))
+
+
 PARTS = ("psi", "collide", "fused", "cluster")
 
 

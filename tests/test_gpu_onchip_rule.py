@@ -34,3 +34,29 @@ def test_auto_takes_the_faster_update(lbm, case):
     sim.set_geometry(np.zeros((batch, nz, ny, nx), np.uint8))
     assert lbm.lbm_resolved_kernel(sim.ctx, n) == ("persistent" if case in ONCHIP else "compact")
     sim.close()
+
+
+def test_library_says_whether_instances_stay_on_chip(lbm):
+    """lbm_resolved_onchip follows the kernel that runs: storage, instance size, number of
+    updates, wall slip, and the failure test of the grid-wide barriers."""
+    def ctx(shape, precision="fp32", kernel="auto", **params):
+        nx, ny, nz = shape
+        sim = lbm.Sim(nx, ny, nz, [dict(tau=(1.0, 1.0), G=-1.8, **params)], precision=precision, kernel=kernel)
+        assert not lbm.lbm_resolved_onchip(sim.ctx, 10)  # no geometry yet
+        sim.set_geometry(np.zeros((1, nz, ny, nx), np.uint8))
+        return sim
+    sim = ctx((20, 20, 20))
+    assert lbm.lbm_resolved_onchip(sim.ctx, 8) and not lbm.lbm_resolved_onchip(sim.ctx, 7)
+    lbm.lbm_set_barrier_test(sim.ctx, 4_000_000_000, 1)
+    assert not lbm.lbm_resolved_onchip(sim.ctx, 8)
+    lbm.lbm_set_barrier_test(sim.ctx, 4_000_000_000, 0)
+    sim.set_params([dict(tau=(1.0, 1.0), slip=0.5)])
+    assert not lbm.lbm_resolved_onchip(sim.ctx, 8)
+    sim.close()
+    for shape, precision, kernel, want in (((32, 16, 16), "fp16s", "persistent", True),
+                                           ((31, 17, 16), "bf16s", "persistent", False),  # 8432 cells
+                                           ((16, 16, 16), "fp64", "persistent", False),
+                                           ((16, 16, 16), "fp32", "compact", False)):
+        sim = ctx(shape, precision, kernel)
+        assert lbm.lbm_resolved_onchip(sim.ctx, 2) == want, (shape, precision, kernel)
+        sim.close()
