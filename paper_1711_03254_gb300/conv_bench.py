@@ -5,9 +5,9 @@
 For every 3x3x3 layer of the U-Net (surrogate.Surrogate's layer table at the
 given resolution and batch) this times, with CUDA events on the current stream
 after warm-up:
-  - the forward convolution with each forward kernel ("resident": the
-    automatic resident choice, "pertile": one block per tile, "persistent":
-    persistent wherever it fits, "gather": the gathered kernel);
+  - the forward convolution with each forward kernel ("auto": the automatic
+    choice, "resident": one block per tile with all output channels,
+    "persistent": persistent wherever it fits, "gather": the gathered kernel);
   - the data gradient (the forward kernel on flipped weights, Ci and Co
     exchanged; the first layer has none);
   - the weight gradient with each of its kernels ("auto": the automatic choice,
@@ -81,7 +81,7 @@ def main(argv=None):
     g = torch.Generator(device=dev)
     g.manual_seed(1)
     peak = _peak()
-    tot = {"fwd_resident": 0.0, "fwd_pertile": 0.0, "fwd_persistent": 0.0, "fwd_gather": 0.0,
+    tot = {"fwd_auto": 0.0, "fwd_resident": 0.0, "fwd_persistent": 0.0, "fwd_gather": 0.0,
            "bwd_data": 0.0, "bwd_weight_auto": 0.0, "bwd_weight_resident": 0.0, "bwd_weight_pairs": 0.0, "bwd_weight_gather": 0.0}
     flops_tot = {"fwd": 0.0, "bwd_data": 0.0, "bwd_weight": 0.0}
     for name, ci, co, s in layers(args.size):
@@ -101,7 +101,7 @@ def main(argv=None):
         prev = ws.ws_conv3d_fwd_algo("auto")
         prev_w = ws.ws_conv3d_bwd_weight_algo("auto")
         try:
-            for algo in ("resident", "pertile", "persistent", "gather"):
+            for algo in ("auto", "resident", "persistent", "gather"):
                 ws.ws_conv3d_fwd_algo(algo)
                 ms = _time(torch, lambda: ws.ws_conv3d_fwd(x, w, b, y, True), args.reps)
                 row[f"fwd_{algo}_ms"] = round(ms, 4)
@@ -126,7 +126,7 @@ def main(argv=None):
         flops_tot["fwd"] += flops
         flops_tot["bwd_weight"] += flops
         if peak:
-            row["fwd_resident_frac"] = round(row["fwd_resident_tflops"] / peak, 3)
+            row["fwd_auto_frac"] = round(row["fwd_auto_tflops"] / peak, 3)
         print(json.dumps(row), flush=True)
     if ws.ws_tc_status() != 0:
         raise RuntimeError("a tensor-core convolution gave up on a bounded wait")

@@ -1464,9 +1464,9 @@ static int sm_count() {
     return n;
 }
 
-// forward kernel choice: 0 automatic, 1 gathered tiles (k_conv_fwd_tc), 2 resident tiles
-// (k_conv3_fwd_pers or k_conv3_fwd_res, as measured faster), 3 resident tiles, one block per tile
-// (k_conv3_fwd_res only), 4 resident tiles, persistent wherever its buffers fit
+// forward kernel choice: 0 automatic (resident tiles, split for small grids), 1 gathered tiles
+// (k_conv_fwd_tc), 2 and 3 resident tiles with all output channels (k_conv3_fwd_res), 4 the same
+// tiles in the persistent kernel (k_conv3_fwd_pers) wherever its buffers fit
 static int g_fwd_algo = 0;
 
 // cuTensorMapEncodeTiled from the driver, fetched through the runtime (no libcuda link)
@@ -1623,44 +1623,35 @@ static bool pers_plan(const ResPlan &res, int Co, ResPlan &p, uint32_t &buf_cols
     return false;
 }
 
-// The persistent forward kernel runs on request only: two or three blocks of one
-// tile each per SM measured as fast or faster on every layer of the U-Net (batch 4,
-// us: 32^3 64->64 45 against 50, 160->64 94 against 114, 16^3 224->96 38 against 43, 64^3
-// 16->32 63 against 85; 32->64 29.6 against 29.0).
-static bool want_persistent() { return g_fwd_algo == 4; }
-
 // Small grids (automatic choice): a plan that leaves SMs idle, or one block per
 // SM where two would share its tensor core, is replaced by one with fewer lines
 // per tile, more resident blocks or the output channels split over nco blocks,
 // when a model of the kernel's time says so by more than 10 %.  The model, in
 // SM clocks, from measurements on GB300 with loads or MMAs left out: an M128 K16
-// MMA takes about 43 + 0.65 N (at least 105 when one block is alone on its SM,
-// because consecutive MMAs on one accumulator wait for each other), TMA 1.5
-// per 32-byte row, both shared by the blocks of an SM, 3000 per round of
-// resident blocks for the start and the epilogue.  Neither choice changes the
-// order of any sum, so the bits stay.  us per call, before and after: 8^3
-// 128->128 20.6, 16.5; 16^3 96->96 21.7, 13.6; 224->96 42.9, 26.6; batch 4, 32^3
-// 160->64 114, 94; 64->64 50, 45.  (At 3 % instead of 10 it also moved 64^3 32->32
-// from 11 lines to 13: 111 us against 103.)
-struct GridCost {
-    double clocks;
-    int per_sm;
-};
-static GridCost grid_cost(const Act &a, int Ci, int N, int nco, int by, int nt, int pitch, int per_sm, bool persistent) {
-    const long long blocks = (long long)a.N * a.D * ((a.H + by - 1) / by) * nco;
-    const long long m = (blocks + sm_count() - 1) / sm_count();  // blocks of the busiest SM
-    const bool alone = m < 2 || persistent || per_sm < 2;
-    const double mma = 9.0 * nt * (alone ? std::max(105.0, 59.0 + 0.65 * N) : 43.0 + 0.65 * N);
-    const double tma = 1.5 * ((by + 2) * pitch + 9.0 * N);
-    const long long rounds = persistent ? 1 : (m + per_sm - 1) / per_sm;
-    return {(double)m * (Ci / 16) * 3.0 * std::max(mma, tma) + 3000.0 * (double)rounds, per_sm};
+// MMA takes 43 + 0.65 N where blocks share the SM, and 59 + 0.65 N but at least
+// 105 where one is alone on it, because consecutive MMAs on one accumulator wait
+// for each other; TMA takes 1.5 per 32-byte row; both are shared by the blocks of
+// an SM, and a round of resident blocks takes 3000 for the start and the
+// epilogue.  Neither choice changes the order of any sum, so the bits stay.  us
+// per call, before and after: 8^3 128->128 20.6, 16.5; 16^3 96->96 21.7, 13.6;
+// 224->96 42.9, 26.6; batch 4, 32^3 160->64 114, 94; 64->64 50, 45.  The 10 % are the
+// model's error: at 3 % one sample of 64^3 32->96 goes from 62.6 to 68.0, while 16^3
+// 96->224 at batch 4 goes from 33.4 to 29.2.
+static double grid_cost(const Act &a, int Ci, int N, int nco, const ResPlan &p, int sms) {
+    const long long blocks = (long long)a.N * a.D * p.nyt * nco;
+    const long long m = (blocks + sms - 1) / sms;  // blocks of the busiest SM
+    const bool alone = m < 2 || p.per_sm < 2;
+    const double mma = 9.0 * p.ntiles * (alone ? std::max(105.0, 59.0 + 0.65 * N) : 43.0 + 0.65 * N);
+    const double tma = 1.5 * ((p.by + 2) * p.pitch + 9.0 * N);
+    const long long rounds = (m + p.per_sm - 1) / p.per_sm;
+    return (double)m * (Ci / 16) * 3.0 * std::max(mma, tma) + 3000.0 * (double)rounds;
 }
-static bool small_grid_plan(const Act &a, int Ci, int Co, const ResPlan &base, bool persistent, ResPlan &out,
-                            int &nco_out) {
+static bool small_grid_plan(const Act &a, int Ci, int Co, int sms, ResPlan &plan, int &nco_out) {
+    const ResPlan base = plan;
     const long long base_blocks = (long long)a.N * a.D * base.nyt;
-    if (base_blocks > 12LL * sm_count()) return false;
+    if (base_blocks > 12LL * sms) return false;
     const int pitch = base.pitch;
-    double best = 0.9 * grid_cost(a, Ci, Co, 1, base.by, base.ntiles, pitch, persistent ? 1 : base.per_sm, persistent).clocks;
+    double best = 0.9 * grid_cost(a, Ci, Co, 1, base, sms);
     bool found = false;
     for (int nco : {1, 2, 3, 4, 6, 8}) {
         if (Co % (16 * nco)) continue;
@@ -1682,7 +1673,7 @@ static bool small_grid_plan(const Act &a, int Ci, int Co, const ResPlan &base, b
             p.a_half = (uint32_t)R * 16u;
             p.stage_bytes = 2 * p.a_half + 18u * (uint32_t)N * 16u;
             p.tx_bytes = 2u * (uint32_t)((by + 2) * pitch) * 16u + 18u * (uint32_t)N * 16u;
-            const long long blocks = (long long)a.N * a.D * p.nyt * nco, m = (blocks + sm_count() - 1) / sm_count();
+            const long long blocks = (long long)a.N * a.D * p.nyt * nco, m = (blocks + sms - 1) / sms;
             // as many resident blocks as the busiest SM has work for, 2 .. 8 stages each
             p.per_sm = (int)std::min<long long>(std::min<long long>(m, 512 / p.cols), 4);
             for (p.stages = 0; p.per_sm >= 1 && !p.stages; p.per_sm -= p.stages ? 0 : 1)
@@ -1694,10 +1685,10 @@ static bool small_grid_plan(const Act &a, int Ci, int Co, const ResPlan &base, b
                     if ((long long)res_smem(q) <= budget) p.stages = ns;
                 }
             if (!p.stages) continue;
-            const double c = grid_cost(a, Ci, N, nco, by, p.ntiles, pitch, p.per_sm, false).clocks;
+            const double c = grid_cost(a, Ci, N, nco, p, sms);
             if (c < best) {
                 best = c;
-                out = p;
+                plan = p;
                 nco_out = nco;
                 found = true;
             }
@@ -1706,71 +1697,80 @@ static bool small_grid_plan(const Act &a, int Ci, int Co, const ResPlan &base, b
     return found;
 }
 
-static int conv3_fwd_res(const void *x, int ldx, const void *w, const float *bias, void *y, int ldy, int y_f32,
-                         const Act &a, int Ci, int Co, int relu, cudaStream_t s, ResPlan pl) {
-    ResPlan pp;
-    uint32_t buf_cols = 0;
-    bool persistent = want_persistent() && pers_plan(pl, Co, pp, buf_cols);
+// What a forward call runs under the current choice on a device of `sms` SMs: the
+// resident plan (of Co / nco output channels a block), or its persistent variant
+// with accumulator buffers of buf_cols columns.  False where no resident plan fits.
+// The persistent kernel runs on request only: two or three blocks of one tile each
+// per SM measured as fast or faster on every layer of the U-Net but one (batch 4,
+// us: 32^3 64->64 45 against 50, 160->64 94 against 114, 16^3 224->96 38 against 43, 64^3
+// 16->32 63 against 85; 32->64 29.6 against 29.0).
+struct FwdPlan {
+    ResPlan res;
     int nco = 1;
-    if (g_fwd_algo == 0) {
-        ResPlan sp;
-        if (small_grid_plan(a, Ci, Co, pl, persistent, sp, nco)) {
-            pl = sp;
-            persistent = false;
-        }
+    bool persistent = false;
+    uint32_t buf_cols = 0;
+    size_t smem = 0;
+    long long grid = 0;
+};
+static bool fwd_choose(const Act &a, int Ci, int Co, int sms, FwdPlan &f) {
+    ResPlan pl, pp;
+    if (g_fwd_algo == 1 || !res_plan(a.W, a.H, Co, pl)) return false;
+    uint32_t buf_cols = 0;
+    if (g_fwd_algo == 4 && pers_plan(pl, Co, pp, buf_cols)) {
+        f.res = pp;
+        f.persistent = true;
+        f.buf_cols = buf_cols;
+        f.smem = std::max(pers_smem(pp), (size_t)kSmemPerSM / 2 - kSmemReserved + 16);
+        f.grid = std::min<long long>((long long)a.N * a.D * pl.nyt, sms);  // at most one per tile
+        return true;
     }
+    if (g_fwd_algo == 0) small_grid_plan(a, Ci, Co, sms, pl, f.nco);
+    f.res = pl;
+    f.smem = res_smem_request(pl);
+    f.grid = (long long)a.N * a.D * pl.nyt * f.nco;
+    return true;
+}
+
+static int conv3_fwd_res(const void *x, int ldx, const void *w, const float *bias, void *y, int ldy, int y_f32,
+                         const Act &a, int Ci, int Co, int relu, cudaStream_t s, const FwdPlan &f) {
+    const ResPlan &pl = f.res;
     EncodeTiledFn enc = encode_tiled();
     CUtensorMap xmap, wmap;
     if (!enc || !act_map(&xmap, x, ldx, a, Ci, 16, pl.pitch, pl.by + 2, CU_TENSOR_MAP_SWIZZLE_32B)) return 2;
-    // the weights as [tap][Co][Ci], 16 channels of all Co for nine taps at a time
+    // the weights as [tap][Co][Ci], 16 channels of a block's output channels for nine taps at a time
     const cuuint32_t ones[3] = {1, 1, 1};
     const cuuint64_t wdim[3] = {(cuuint64_t)Ci, (cuuint64_t)Co, 27};
     const cuuint64_t wstr[2] = {(cuuint64_t)Ci * 2 * 27, (cuuint64_t)Ci * 2};
-    const cuuint32_t wbox[3] = {16, (cuuint32_t)(Co / nco), 9};
+    const cuuint32_t wbox[3] = {16, (cuuint32_t)(Co / f.nco), 9};
     if (enc(&wmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(w), wdim, wstr, wbox, ones,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return 2;
-    const size_t smem = res_smem_request(pl);
-    static size_t attr[2] = {0, 0};
-    const int which = y_f32 ? 1 : 0;
-    if (attr[which] < smem) {
-        const cudaError_t e = y_f32 ? cudaFuncSetAttribute(k_conv3_fwd_res<true>,
-                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                                    : cudaFuncSetAttribute(k_conv3_fwd_res<false>,
-                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return 2;
-        attr[which] = smem;
+    const long long tiles = (long long)a.N * a.D * pl.nyt;
+    if (tiles > 0x7FFFFFFFLL || f.grid > 0x7FFFFFFFLL) return 1;
+    const void *fn = f.persistent ? (y_f32 ? (const void *)k_conv3_fwd_pers<true> : (const void *)k_conv3_fwd_pers<false>)
+                                  : (y_f32 ? (const void *)k_conv3_fwd_res<true> : (const void *)k_conv3_fwd_res<false>);
+    static size_t attr[4] = {0, 0, 0, 0};
+    size_t &have = attr[(f.persistent ? 2 : 0) + (y_f32 ? 1 : 0)];
+    if (have < f.smem) {
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f.smem) != cudaSuccess) return 2;
+        have = f.smem;
     }
-    const long long blocks = (long long)a.N * a.D * pl.nyt * nco;
-    if (blocks > 0x7FFFFFFFLL) return 1;
-    if (persistent) {
-        // one persistent block per SM (at most one per tile)
-        const size_t psmem = std::max(pers_smem(pp), (size_t)kSmemPerSM / 2 - kSmemReserved + 16);
-        static size_t pattr[2] = {0, 0};
-        if (pattr[which] < psmem) {
-            const cudaError_t e = y_f32 ? cudaFuncSetAttribute(k_conv3_fwd_pers<true>,
-                                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psmem)
-                                        : cudaFuncSetAttribute(k_conv3_fwd_pers<false>,
-                                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psmem);
-            if (e != cudaSuccess) return 2;
-            pattr[which] = psmem;
-        }
-        const unsigned grid = (unsigned)std::min<long long>(blocks, sm_count());
+    const unsigned grid = (unsigned)f.grid;
+    if (f.persistent) {
         if (y_f32)
-            k_conv3_fwd_pers<true><<<grid, PTHREADS, psmem, s>>>(xmap, wmap, bias, y, ldy, a, Ci, Co, relu, pp,
-                                                                 (int)blocks, buf_cols);
+            k_conv3_fwd_pers<true><<<grid, PTHREADS, f.smem, s>>>(xmap, wmap, bias, y, ldy, a, Ci, Co, relu, pl,
+                                                                  (int)tiles, f.buf_cols);
         else
-            k_conv3_fwd_pers<false><<<grid, PTHREADS, psmem, s>>>(xmap, wmap, bias, y, ldy, a, Ci, Co, relu, pp,
-                                                                  (int)blocks, buf_cols);
-        return cudaGetLastError() == cudaSuccess ? 0 : 2;
+            k_conv3_fwd_pers<false><<<grid, PTHREADS, f.smem, s>>>(xmap, wmap, bias, y, ldy, a, Ci, Co, relu, pl,
+                                                                   (int)tiles, f.buf_cols);
+    } else if (y_f32) {
+        k_conv3_fwd_res<true><<<grid, RTHREADS, f.smem, s>>>(xmap, wmap, bias, y, ldy, a, Ci, Co / f.nco, f.nco, relu,
+                                                             pl);
+    } else {
+        k_conv3_fwd_res<false><<<grid, RTHREADS, f.smem, s>>>(xmap, wmap, bias, y, ldy, a, Ci, Co / f.nco, f.nco, relu,
+                                                              pl);
     }
-    if (y_f32)
-        k_conv3_fwd_res<true><<<(unsigned)blocks, RTHREADS, smem, s>>>(xmap, wmap, bias, y, ldy, a, Ci, Co / nco, nco,
-                                                                       relu, pl);
-    else
-        k_conv3_fwd_res<false><<<(unsigned)blocks, RTHREADS, smem, s>>>(xmap, wmap, bias, y, ldy, a, Ci, Co / nco, nco,
-                                                                        relu, pl);
     return cudaGetLastError() == cudaSuccess ? 0 : 2;
 }
 
@@ -1789,6 +1789,30 @@ constexpr int kWgWaves = 1;
 
 static size_t wg_smem(const WgPlan &p) { return (size_t)p.stages * p.stage_bytes + 1024 + 8 * (2 * p.stages + 2) + 16; }
 
+// the most stages (2 .. 4) at the most blocks per SM that the plan's tensor-memory
+// columns allow: sets the stages and returns the blocks per SM, 0 where not even two fit
+static int wg_stages(WgPlan &p) {
+    for (int per_sm = 512 / p.cols; per_sm >= 1; --per_sm) {
+        const long long budget = std::min((long long)kSmemPerSM / per_sm - kSmemReserved, (long long)kSmemPerBlockMax);
+        for (p.stages = 4; p.stages >= 2; --p.stages)
+            if ((long long)wg_smem(p) <= budget) return per_sm;
+    }
+    return 0;
+}
+
+// K-blocks of a plan whose lines are set, shared out over position blocks so that
+// the launch (by_blocks blocks per position block) has kWgWaves full waves; false
+// where the counts do not fit a launch
+static bool wg_split(const Act &a, WgPlan &p, int by_blocks, int resident, int sms) {
+    p.nyb = (a.H + p.by - 1) / p.by;
+    const long long nkb = (long long)a.N * a.D * p.nyb;
+    if (nkb > 0x7FFFFFFFLL) return false;
+    const long long npb = std::min(nkb, std::max(1LL, (long long)kWgWaves * resident * sms / by_blocks));
+    p.kpb = (int)((nkb + npb - 1) / npb);
+    p.npb = (int)((nkb + p.kpb - 1) / p.kpb);
+    return by_blocks <= 65535;
+}
+
 // Plan of k_conv3_wgrad_res: the widest channel block (128, 64, 32 or 16
 // channels dividing Ci; M = 128 rows hold 128 / ci_blk tap pairs), K-blocks
 // of at most 132 rows (whole lines of W + 2 columns; the best of 2 .. 12 lines
@@ -1796,7 +1820,7 @@ static size_t wg_smem(const WgPlan &p) { return (size_t)p.stages * p.stage_bytes
 // stages (2 .. 4) at the most blocks per SM that the tensor memory (3 Co
 // columns) allows, and kWgWaves full waves of blocks in all.  Returns false
 // where no plan fits (W > 254, Co > 160, or not even two stages).
-static bool wg_plan(const Act &a, int Ci, int Co, WgPlan &p) {
+static bool wg_plan(const Act &a, int Ci, int Co, int sms, WgPlan &p) {
     const int pitch = a.W + 2;
     if (pitch > 256 || 3 * Co > 512) return false;
     int cb = 128;
@@ -1808,38 +1832,17 @@ static bool wg_plan(const Act &a, int Ci, int Co, WgPlan &p) {
     p.pitch = pitch;
     p.cols = 32;
     while (p.cols < 3 * Co) p.cols *= 2;
-    bool found = false;
-    int resident = 1;
-    for (int by = std::max(1, std::min(a.H, 132 / pitch)); by >= 1 && !found; --by) {
+    int resident = 0;
+    for (int by = std::max(1, std::min(a.H, 132 / pitch)); by >= 1 && !resident; --by) {
         p.by = by;
         p.ksteps = (by * pitch + 15) / 16;
         const int rb = (p.ksteps * 16 + 2 + 7) / 8 * 8;
         p.region = (uint32_t)rb * 16u;
         p.stage_bytes = (uint32_t)(16 + Co / 8) * p.region;
-        for (int per_sm = 512 / p.cols; per_sm >= 1 && !found; --per_sm) {
-            long long budget = (long long)kSmemPerSM / per_sm - kSmemReserved;
-            if (budget > kSmemPerBlockMax) budget = kSmemPerBlockMax;
-            for (int ns = 4; ns >= 2; --ns) {
-                p.stages = ns;
-                if ((long long)wg_smem(p) <= budget) {
-                    found = true;
-                    resident = per_sm;
-                    break;
-                }
-            }
-        }
+        resident = wg_stages(p);
     }
-    if (!found) return false;
-    p.nyb = (a.H + p.by - 1) / p.by;
-    const long long nkb = (long long)a.N * a.D * p.nyb;
-    if (nkb > 0x7FFFFFFFLL) return false;
-    const int by_blocks = (Ci / cb) * p.ntile;
-    long long npb = (long long)kWgWaves * resident * sm_count() / by_blocks;  // no partial last wave
-    if (npb < 1) npb = 1;
-    if (npb > nkb) npb = nkb;
-    p.kpb = (int)((nkb + npb - 1) / npb);
-    p.npb = (int)((nkb + p.kpb - 1) / p.kpb);
-    return by_blocks <= 65535;
+    if (!resident) return false;
+    return wg_split(a, p, (Ci / cb) * p.ntile, resident, sms);
 }
 
 // Plan of k_conv3_wgrad_dz (Ci a multiple of 32, Co <= 48): K-blocks of at
@@ -1847,7 +1850,7 @@ static bool wg_plan(const Act &a, int Ci, int Co, WgPlan &p) {
 // two halo lines and the rows the dy, dx shifts reach past the last K-step,
 // the most stages (2 .. 4) that fit at the blocks per SM the tensor memory
 // (9 Co columns) allows, kWgWaves full waves of blocks in all.
-static bool wg_dz_plan(const Act &a, int Ci, int Co, WgPlan &p) {
+static bool wg_dz_plan(const Act &a, int Ci, int Co, int sms, WgPlan &p) {
     const int pitch = a.W + 2;
     if (pitch > 256 || Ci % 32 || Co > 48) return false;
     p.ci_blk = 32;
@@ -1857,46 +1860,25 @@ static bool wg_dz_plan(const Act &a, int Ci, int Co, WgPlan &p) {
     p.cols = 32;
     while (p.cols < 9 * Co) p.cols *= 2;
     const int nreg = std::max(16, 13 + Co / 8);
-    bool found = false;
-    int resident = 1;
-    for (int by = std::max(1, std::min(a.H, 132 / pitch)); by >= 1 && !found; --by) {
+    int resident = 0;
+    for (int by = std::max(1, std::min(a.H, 132 / pitch)); by >= 1 && !resident; --by) {
         if (by + 2 > 256) continue;
         p.by = by;
         p.ksteps = (by * pitch + 15) / 16;
         const int rb = (std::max((by + 2) * pitch, p.ksteps * 16 + 2 * pitch + 2) + 7) / 8 * 8;
         p.region = (uint32_t)rb * 16u;
         p.stage_bytes = (uint32_t)nreg * p.region;
-        for (int per_sm = 512 / p.cols; per_sm >= 1 && !found; --per_sm) {
-            long long budget = (long long)kSmemPerSM / per_sm - kSmemReserved;
-            if (budget > kSmemPerBlockMax) budget = kSmemPerBlockMax;
-            for (int ns = 4; ns >= 2; --ns) {
-                p.stages = ns;
-                if ((long long)wg_smem(p) <= budget) {
-                    found = true;
-                    resident = per_sm;
-                    break;
-                }
-            }
-        }
+        resident = wg_stages(p);
     }
-    if (!found) return false;
-    p.nyb = (a.H + p.by - 1) / p.by;
-    const long long nkb = (long long)a.N * a.D * p.nyb;
-    if (nkb > 0x7FFFFFFFLL) return false;
-    const int by_blocks = Ci / 32;
-    long long npb = (long long)kWgWaves * resident * sm_count() / by_blocks;  // no partial last wave
-    if (npb < 1) npb = 1;
-    if (npb > nkb) npb = nkb;
-    p.kpb = (int)((nkb + npb - 1) / npb);
-    p.npb = (int)((nkb + p.kpb - 1) / p.kpb);
-    return by_blocks <= 65535;
+    if (!resident) return false;
+    return wg_split(a, p, Ci / 32, resident, sms);
 }
 
 // Plan of k_conv3_wgrad_dz with three copies of dY (same conditions): as
 // wg_dz_plan, with X groups of (by + 2) lines and the rows the dy shift of the
 // last K-step reaches, dY groups of whole K-steps, and stages that also cover
 // what the eighth M group (dropped rows) reads.  `region` is half an X group.
-static bool wg_copies_plan(const Act &a, int Ci, int Co, WgPlan &p) {
+static bool wg_copies_plan(const Act &a, int Ci, int Co, int sms, WgPlan &p) {
     const int pitch = a.W + 2;
     if (pitch > 256 || Ci % 32 || Co > 48) return false;
     p.ci_blk = 32;
@@ -1905,9 +1887,8 @@ static bool wg_copies_plan(const Act &a, int Ci, int Co, WgPlan &p) {
     p.pitch = pitch;
     p.cols = 32;
     while (p.cols < 9 * Co) p.cols *= 2;
-    bool found = false;
-    int resident = 1;
-    for (int by = std::max(1, std::min(a.H, 132 / pitch)); by >= 1 && !found; --by) {
+    int resident = 0;
+    for (int by = std::max(1, std::min(a.H, 132 / pitch)); by >= 1 && !resident; --by) {
         if (by + 2 > 256) continue;
         p.by = by;
         p.ksteps = (by * pitch + 15) / 16;
@@ -1915,38 +1896,18 @@ static bool wg_copies_plan(const Act &a, int Ci, int Co, WgPlan &p) {
         p.region = (uint32_t)rb * 16u;
         const uint32_t gy = (uint32_t)p.ksteps * 512u;
         p.stage_bytes = std::max(12 * p.region + (1 + 3 * (uint32_t)(Co / 16)) * gy, 16 * p.region);
-        for (int per_sm = 512 / p.cols; per_sm >= 1 && !found; --per_sm) {
-            long long budget = (long long)kSmemPerSM / per_sm - kSmemReserved;
-            if (budget > kSmemPerBlockMax) budget = kSmemPerBlockMax;
-            for (int ns = 4; ns >= 2; --ns) {
-                p.stages = ns;
-                if ((long long)wg_smem(p) <= budget) {
-                    found = true;
-                    resident = per_sm;
-                    break;
-                }
-            }
-        }
+        resident = wg_stages(p);
     }
-    if (!found) return false;
-    p.nyb = (a.H + p.by - 1) / p.by;
-    const long long nkb = (long long)a.N * a.D * p.nyb;
-    if (nkb > 0x7FFFFFFFLL) return false;
-    const int by_blocks = Ci / 32;
-    long long npb = (long long)kWgWaves * resident * sm_count() / by_blocks;  // no partial last wave
-    if (npb < 1) npb = 1;
-    if (npb > nkb) npb = nkb;
-    p.kpb = (int)((nkb + npb - 1) / npb);
-    p.npb = (int)((nkb + p.kpb - 1) / p.kpb);
-    return by_blocks <= 65535;
+    if (!resident) return false;
+    return wg_split(a, p, Ci / 32, resident, sms);
 }
 
 // weight-gradient kernels with resident tiles, and the plan of the one a call runs under the current choice
 enum WgKernel { kWgPairs = 0, kWgDz = 1, kWgCopies = 2, kWgNone = -1 };
-static WgKernel wg_choose(const Act &a, int Ci, int Co, WgPlan &p) {
-    if (g_wgrad_algo == 0 && wg_copies_plan(a, Ci, Co, p)) return kWgCopies;
-    if (g_wgrad_algo != 3 && wg_dz_plan(a, Ci, Co, p)) return kWgDz;
-    return wg_plan(a, Ci, Co, p) ? kWgPairs : kWgNone;
+static WgKernel wg_choose(const Act &a, int Ci, int Co, int sms, WgPlan &p) {
+    if (g_wgrad_algo == 0 && wg_copies_plan(a, Ci, Co, sms, p)) return kWgCopies;
+    if (g_wgrad_algo != 3 && wg_dz_plan(a, Ci, Co, sms, p)) return kWgDz;
+    return wg_plan(a, Ci, Co, sms, p) ? kWgPairs : kWgNone;
 }
 
 static size_t wg_smem_request(const WgPlan &p) {
@@ -1997,8 +1958,9 @@ int ws_conv3d_fwd(const void *x, int ldx, const void *w, const float *bias, void
     const long long P = (long long)N * D * H * W;
     cudaStream_t s = (cudaStream_t)stream;
     if (k == 3 && g_fwd_algo != 1) {
-        ResPlan pl;
-        if (res_plan(W, H, Co, pl)) return conv3_fwd_res(x, ldx, w, bias, y, ldy, y_f32, a, Ci, Co, relu, s, pl);
+        FwdPlan f;
+        if (fwd_choose(a, Ci, Co, sm_count(), f))
+            return conv3_fwd_res(x, ldx, w, bias, y, ldy, y_f32, a, Ci, Co, relu, s, f);
         if (g_fwd_algo >= 2) return 1;
     }
     const long long head_blocks = (P + kHeadThreads - 1) / kHeadThreads;
@@ -2037,37 +1999,25 @@ int ws_conv3d_fwd_algo(int algo) {
     return prev;
 }
 
-int ws_conv3d_plan(int which, int N, int D, int H, int W, int Ci, int Co, long long *out, int nout) {
-    if (!out || nout < 0 || N < 1 || D < 1 || H < 1 || W < 1 || bad_channels(Ci) || bad_channels(Co) || Co > 256 ||
-        (which != 0 && which != 1))
+int ws_conv3d_plan_for(int sms, int which, int N, int D, int H, int W, int Ci, int Co, long long *out, int nout) {
+    if (sms < 1 || !out || nout < 0 || N < 1 || D < 1 || H < 1 || W < 1 || bad_channels(Ci) || bad_channels(Co) ||
+        Co > 256 || (which != 0 && which != 1))
         return -2;
     long long v[16] = {0};
     int n = 0;
     const Act a{N, D, H, W};
     if (which == 0) {
-        ResPlan pl, pp;
-        uint32_t buf_cols = 0;
-        if (g_fwd_algo == 1 || !res_plan(W, H, Co, pl)) return -1;
-        const long long tiles = (long long)N * D * pl.nyt;
-        bool pers = want_persistent() && pers_plan(pl, Co, pp, buf_cols);
-        ResPlan sp;
-        int nco = 1;
-        if (g_fwd_algo == 0 && small_grid_plan(a, Ci, Co, pl, pers, sp, nco)) {
-            pl = sp;
-            pers = false;
-        }
-        const ResPlan &q = pers ? pp : pl;
-        const size_t smem = pers ? std::max(pers_smem(pp), (size_t)kSmemPerSM / 2 - kSmemReserved + 16)
-                                 : res_smem_request(pl);
-        const long long f[14] = {pers ? 1 : 0, q.by, q.nyt, q.pitch, q.ntiles, q.stages, q.cols, q.per_sm,
-                                 q.a_half, q.stage_bytes, q.tx_bytes, (long long)smem,
-                                 pers ? std::min<long long>(tiles, sm_count()) : (long long)N * D * pl.nyt * nco,
-                                 pers ? (long long)buf_cols : 0};
-        for (; n < 14; ++n) v[n] = f[n];
+        FwdPlan p;
+        if (!fwd_choose(a, Ci, Co, sms, p)) return -1;
+        const ResPlan &q = p.res;
+        const long long f[15] = {p.persistent ? 1 : 0, q.by, q.nyt, q.pitch, q.ntiles, q.stages, q.cols, q.per_sm,
+                                 q.a_half, q.stage_bytes, q.tx_bytes, (long long)p.smem, p.grid, (long long)p.buf_cols,
+                                 p.nco};
+        for (; n < 15; ++n) v[n] = f[n];
     } else {
         WgPlan pl;
         if (g_wgrad_algo == 1) return -1;
-        const WgKernel kind = wg_choose(a, Ci, Co, pl);
+        const WgKernel kind = wg_choose(a, Ci, Co, sms, pl);
         if (kind == kWgNone) return -1;
         const long long f[16] = {kind, pl.by, pl.nyb, pl.pitch, pl.ksteps, pl.J, pl.ci_blk, pl.ntile,
                                  pl.npb, pl.kpb, pl.stages, pl.cols, pl.region, pl.stage_bytes,
@@ -2076,6 +2026,10 @@ int ws_conv3d_plan(int which, int N, int D, int H, int W, int Ci, int Co, long l
     }
     for (int i = 0; i < n && i < nout; ++i) out[i] = v[i];
     return n;
+}
+
+int ws_conv3d_plan(int which, int N, int D, int H, int W, int Ci, int Co, long long *out, int nout) {
+    return ws_conv3d_plan_for(sm_count(), which, N, D, H, W, Ci, Co, out, nout);
 }
 
 int ws_conv3d_bwd_weight_algo(int algo) {
@@ -2120,7 +2074,7 @@ int ws_conv3d_bwd_weight(const void *x, int ldx, const void *dy, int ldy, float 
     if (k == 3 && g_wgrad_algo != 1) {
         WgPlan pl;
         // Ci a multiple of 32 and Co <= 48: the dz-slot kernel (each X line loaded 3 times, not 9)
-        const WgKernel kind = wg_choose(a, Ci, Co, pl);
+        const WgKernel kind = wg_choose(a, Ci, Co, sm_count(), pl);
         if (kind != kWgNone) {
             // the kernel sums the bias gradient too when it has a free slot for a row of ones
             const bool fold = db && (kind != kWgPairs || pl.J * pl.ntile > 9);

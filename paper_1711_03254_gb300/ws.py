@@ -23,6 +23,7 @@ def _lib():
         L.ws_conv3d_fwd_algo.argtypes = [i]
         L.ws_conv3d_bwd_weight_algo.argtypes = [i]
         L.ws_conv3d_plan.argtypes = [i, i, i, i, i, i, i, ctypes.POINTER(ll), i]
+        L.ws_conv3d_plan_for.argtypes = [i, i, i, i, i, i, i, i, ctypes.POINTER(ll), i]
         L.ws_conv3d_flip_weights.argtypes = [vp, vp, i, i, i, vp]
         L.ws_conv3d_bwd_weight.argtypes = [vp, i, vp, i, vp, vp, i, i, i, i, i, i, i, vp]
         L.ws_avgpool2.argtypes = [vp, i, vp, i, i, i, i, i, i, vp]
@@ -37,7 +38,7 @@ def _lib():
         for name in ("ws_conv3d_fwd", "ws_conv3d_fwd_algo", "ws_conv3d_flip_weights", "ws_conv3d_bwd_weight",
                      "ws_conv3d_bwd_weight_algo", "ws_avgpool2", "ws_avgpool2_bwd", "ws_upsample2",
                      "ws_upsample2_bwd", "ws_relu_bwd", "ws_mse_loss", "ws_adam",
-                     "ws_to_bf16", "ws_tc_status", "ws_conv3d_plan"):
+                     "ws_to_bf16", "ws_tc_status", "ws_conv3d_plan", "ws_conv3d_plan_for"):
             getattr(L, name).restype = ctypes.c_int
         _sig_done = True
     return L
@@ -80,9 +81,9 @@ def ws_conv3d_fwd(x, w, bias, y, relu: bool):
 
 def ws_conv3d_fwd_algo(algo: str) -> str:
     """Forward kernel of later ws_conv3d_fwd calls: "auto", "gather",
-    "resident", "pertile" (resident, one block per tile, never persistent) or
-    "persistent" (resident, persistent wherever its buffers fit); returns the
-    previous choice."""
+    "resident" (one block per tile, with all output channels), "pertile" (the
+    same) or "persistent" (resident, persistent wherever its buffers fit);
+    returns the previous choice."""
     names = ("auto", "gather", "resident", "pertile", "persistent")
     prev = _lib().ws_conv3d_fwd_algo(names.index(algo))
     if prev < 0:
@@ -102,23 +103,32 @@ def ws_conv3d_bwd_weight_algo(algo: str) -> str:
 
 
 _FWD_PLAN = ("persistent", "by", "nyt", "pitch", "ntiles", "stages", "cols", "per_sm", "a_half", "stage_bytes",
-             "tx_bytes", "smem", "grid", "buf_cols")
+             "tx_bytes", "smem", "grid", "buf_cols", "nco")
 _WGRAD_PLAN = ("dz", "by", "nyb", "pitch", "ksteps", "J", "ci_blk", "ntile", "npb", "kpb", "stages", "cols",
                "region", "stage_bytes", "smem", "grid_y")
+
+
+def _plan(query, which, *args):
+    names = _FWD_PLAN if which == "fwd" else _WGRAD_PLAN
+    out = (ctypes.c_longlong * 16)()
+    n = query(0 if which == "fwd" else 1, *args, out, 16)
+    if n == -1:
+        return None
+    if n < 0:
+        raise WsError(f"ws_conv3d_plan rejected {which} {args}")
+    return dict(zip(names, out[:n]))
 
 
 def ws_conv3d_plan(which: str, N: int, D: int, H: int, W: int, Ci: int, Co: int):
     """Tiling of the resident-tile kernels for a 3x3x3 convolution ("fwd" or
     "wgrad") under the current kernel choice, as a dict; None where the
     gathered kernel would run.  Host only."""
-    names = _FWD_PLAN if which == "fwd" else _WGRAD_PLAN
-    out = (ctypes.c_longlong * 16)()
-    n = _lib().ws_conv3d_plan(0 if which == "fwd" else 1, N, D, H, W, Ci, Co, out, 16)
-    if n == -1:
-        return None
-    if n < 0:
-        raise WsError(f"ws_conv3d_plan rejected {which} {(N, D, H, W, Ci, Co)}")
-    return dict(zip(names, out[:n]))
+    return _plan(_lib().ws_conv3d_plan, which, N, D, H, W, Ci, Co)
+
+
+def ws_conv3d_plan_for(sms: int, which: str, N: int, D: int, H: int, W: int, Ci: int, Co: int):
+    """ws_conv3d_plan for a device of `sms` SMs."""
+    return _plan(lambda *a: _lib().ws_conv3d_plan_for(sms, *a), which, N, D, H, W, Ci, Co)
 
 
 def ws_conv3d_flip_weights(w, wf):
