@@ -1507,6 +1507,11 @@ static int res_tiles(int lt, int pitch, int W) { return ((lt - 1) * pitch + W + 
 // keep the search's stages and blocks per SM.  Returns false if none fits.
 static constexpr int kSmemPerSM = 233472, kSmemPerBlockMax = 232448, kSmemReserved = 1024;
 static size_t res_smem(const ResPlan &p) { return (size_t)p.stages * p.stage_bytes + 1024 + 8 * (2 * p.stages + 2) + 16; }
+// stages of `stage_bytes` that fit each of per_sm blocks (the inverse of res_smem)
+static int res_stages(uint32_t stage_bytes, int per_sm) {
+    const int budget = std::min(kSmemPerSM / per_sm - kSmemReserved, kSmemPerBlockMax);
+    return (budget - 1056) / (int)(stage_bytes + 16);
+}
 static bool res_plan(int W, int H, int Co, ResPlan &best) {
     const int pitch = W + 2;
     if (pitch > 256 || Co > 256) return false;
@@ -1632,8 +1637,9 @@ static bool pers_plan(const ResPlan &res, int Co, ResPlan &p, uint32_t &buf_cols
 // 105 where one is alone on it, because consecutive MMAs on one accumulator wait
 // for each other; TMA takes 1.5 per 32-byte row; both are shared by the blocks of
 // an SM, and a round of resident blocks takes 3000 for the start and the
-// epilogue.  Neither choice changes the order of any sum, so the bits stay.  us
-// per call, before and after: 8^3 128->128 20.6, 16.5; 16^3 96->96 21.7, 13.6;
+// epilogue.  Neither choice changes the order of any sum, so the bits stay.  The search
+// is kept short, because calls of a small grid are bound by their host time (it took
+// 1.2 to 2.7 us, now 0.1 to 0.9).  us per call, before and after: 8^3 128->128 20.6, 16.5; 16^3 96->96 21.7, 13.6;
 // 224->96 42.9, 26.6; batch 4, 32^3 160->64 114, 94; 64->64 50, 45.  The 10 % are the
 // model's error: at 3 % one sample of 64^3 32->96 goes from 62.6 to 68.0, while 16^3
 // 96->224 at batch 4 goes from 33.4 to 29.2.
@@ -1653,38 +1659,36 @@ static bool small_grid_plan(const Act &a, int Ci, int Co, int sms, ResPlan &plan
     const int pitch = base.pitch;
     double best = 0.9 * grid_cost(a, Ci, Co, 1, base, sms);
     bool found = false;
+    const int ly_max = std::min(a.H, 254);
     for (int nco : {1, 2, 3, 4, 6, 8}) {
         if (Co % (16 * nco)) continue;
         const int N = Co / nco;
-        for (int want = 1; want * N <= 512; ++want) {
-            int by = (128 * want - a.W) / pitch + 1;
-            if (128 * want < a.W || by < 1) continue;
-            by = std::min(std::min(by, a.H), 254);
-            const int nyt = (a.H + by - 1) / by;
-            by = (a.H + nyt - 1) / nyt;  // the same tiles per plane, evenly
+        // tile counts that hold a line; the last one that matters holds the whole plane
+        int last_by = 0;
+        for (int want = (a.W + 127) / 128; want * N <= 512 && last_by < ly_max; ++want) {
             ResPlan p;
-            p.by = by;
-            p.nyt = (a.H + by - 1) / by;
+            p.by = std::min((128 * want - a.W) / pitch + 1, ly_max);
+            p.nyt = (a.H + p.by - 1) / p.by;
+            p.by = (a.H + p.nyt - 1) / p.nyt;  // the same tiles per plane, evenly
+            if (p.by == last_by) continue;
+            last_by = p.by;
+            p.nyt = (a.H + p.by - 1) / p.by;
             p.pitch = pitch;
-            p.ntiles = res_tiles(by, pitch, a.W);
+            p.ntiles = res_tiles(p.by, pitch, a.W);
             p.cols = 32;
             while (p.cols < p.ntiles * N) p.cols *= 2;
-            const int R = (std::max(128 * p.ntiles + 2 * pitch + 2, (by + 2) * pitch) + 7) / 8 * 8;
+            const int R = (std::max(128 * p.ntiles + 2 * pitch + 2, (p.by + 2) * pitch) + 7) / 8 * 8;
             p.a_half = (uint32_t)R * 16u;
             p.stage_bytes = 2 * p.a_half + 18u * (uint32_t)N * 16u;
-            p.tx_bytes = 2u * (uint32_t)((by + 2) * pitch) * 16u + 18u * (uint32_t)N * 16u;
+            p.tx_bytes = 2u * (uint32_t)((p.by + 2) * pitch) * 16u + 18u * (uint32_t)N * 16u;
             const long long blocks = (long long)a.N * a.D * p.nyt * nco, m = (blocks + sms - 1) / sms;
             // as many resident blocks as the busiest SM has work for, 2 .. 8 stages each
             p.per_sm = (int)std::min<long long>(std::min<long long>(m, 512 / p.cols), 4);
-            for (p.stages = 0; p.per_sm >= 1 && !p.stages; p.per_sm -= p.stages ? 0 : 1)
-                for (int ns = 8; ns >= 2 && !p.stages; --ns) {
-                    ResPlan q = p;
-                    q.stages = ns;
-                    const long long budget =
-                        std::min((long long)kSmemPerSM / p.per_sm - kSmemReserved, (long long)kSmemPerBlockMax);
-                    if ((long long)res_smem(q) <= budget) p.stages = ns;
-                }
-            if (!p.stages) continue;
+            for (p.stages = 0; p.per_sm >= 1; --p.per_sm) {
+                p.stages = std::min(8, res_stages(p.stage_bytes, p.per_sm));
+                if (p.stages >= 2) break;
+            }
+            if (p.per_sm < 1) continue;
             const double c = grid_cost(a, Ci, N, nco, p, sms);
             if (c < best) {
                 best = c;
