@@ -1350,21 +1350,22 @@ __global__ void __launch_bounds__(RTHREADS) k_conv3_wgrad_dz(const __grid_consta
 // dW[co][t][ci] += sum over the nk chunks of part[chunk][t * Ci + ci][co] in a
 // fixed order: per element, lane j = threadIdx.y adds the chunks c = j, j + 8, ...
 // in turn and the eight lane sums are added in lane order, so the result does
-// not depend on scheduling.  A block sums 8 consecutive rows (channels of one tap)
+// not depend on scheduling.  A block sums ROWS consecutive rows (channels of one tap)
 // x 32 output channels: the reads run along co, and the sums are turned in
 // shared memory so that the updates of dW cover whole 32-byte sectors (one
 // element per thread and scattered updates took 33 us for 20 chunks of 160 -> 64
 // channels, 9.4 for 152 of 32 -> 32).  Blocks past the rows (bpart given) add the
 // bias partials, db[co] += sum over nb of bpart[b][co], the same way.
-constexpr int kSumLanes = 8, kSumRows = 8;
+constexpr int kSumLanes = 8;
+template <int ROWS>
 __global__ void __launch_bounds__(32 * kSumLanes) k_wgrad_sum(const float *__restrict__ part, int nk, int rows_pad,
                                                               int rows, int Co, int KV, int Ci,
                                                               float *__restrict__ dW,
                                                               const float *__restrict__ bpart, int nb,
                                                               float *__restrict__ db) {
-    __shared__ float sh[kSumLanes][kSumRows][33];
+    __shared__ float sh[kSumLanes][ROWS][33];
     const int lx = threadIdx.x, j = threadIdx.y, co = (int)blockIdx.y * 32 + lx;
-    const int r0 = (int)blockIdx.x * kSumRows;
+    const int r0 = (int)blockIdx.x * ROWS;
     if (r0 >= rows) {  // the bias
         float s = 0.f;
         if (co < Co)
@@ -1379,22 +1380,22 @@ __global__ void __launch_bounds__(32 * kSumLanes) k_wgrad_sum(const float *__res
         }
         return;
     }
-    float s[kSumRows];
+    float s[ROWS];
 #pragma unroll
-    for (int r = 0; r < kSumRows; ++r) s[r] = 0.f;
+    for (int r = 0; r < ROWS; ++r) s[r] = 0.f;
     if (co < Co) {
         const float *p = part + (size_t)r0 * Co + co;
-#pragma unroll 2
+#pragma unroll (ROWS == 8 ? 2 : 4)
         for (int c = j; c < nk; c += kSumLanes)
 #pragma unroll
-            for (int r = 0; r < kSumRows; ++r) s[r] += p[((size_t)c * rows_pad + r) * Co];
+            for (int r = 0; r < ROWS; ++r) s[r] += p[((size_t)c * rows_pad + r) * Co];
     }
 #pragma unroll
-    for (int r = 0; r < kSumRows; ++r) sh[j][r][lx] = s[r];
+    for (int r = 0; r < ROWS; ++r) sh[j][r][lx] = s[r];
     __syncthreads();
     // one element per thread, rows fastest
-    const int e = j * 32 + lx, r = e % kSumRows, cl = e / kSumRows, cw = (int)blockIdx.y * 32 + cl;
-    if (cw < Co) {
+    const int e = j * 32 + lx, r = e % ROWS, cl = e / ROWS, cw = (int)blockIdx.y * 32 + cl;
+    if (cl < 32 && cw < Co) {
         float t = 0.f;
 #pragma unroll
         for (int l = 0; l < kSumLanes; ++l) t += sh[l][r][cl];
@@ -1402,10 +1403,19 @@ __global__ void __launch_bounds__(32 * kSumLanes) k_wgrad_sum(const float *__res
         dW[((long long)cw * KV + tap) * Ci + ci] += t;
     }
 }
+// 8 rows a block where that makes 350 blocks or more, else 4 with twice the chunks in
+// flight: a block waits for its chunks one after the other, and few blocks leave SMs
+// idle (weight gradient of 32^3 16->16 22.9 us with 8 rows, 16.9 with 4; 64^3 32->32 43.4
+// and 37.4; the other way round 32^3 128->128 51.6 and 54.6).
 static void launch_wgrad_sum(const float *part, int nk, int rows_pad, int rows, int Co, int KV, int Ci, float *dw,
                              const float *bpart, int nb, float *db, cudaStream_t s) {
-    const dim3 grid((unsigned)(rows / kSumRows + (db ? 1 : 0)), (unsigned)((Co + 31) / 32), 1);
-    k_wgrad_sum<<<grid, dim3(32, kSumLanes), 0, s>>>(part, nk, rows_pad, rows, Co, KV, Ci, dw, bpart, nb, db);
+    const unsigned groups = (unsigned)((Co + 31) / 32);
+    auto launch = [&](auto fn, int r) {
+        fn<<<dim3((unsigned)(rows / r + (db ? 1 : 0)), groups, 1), dim3(32, kSumLanes), 0, s>>>(
+            part, nk, rows_pad, rows, Co, KV, Ci, dw, bpart, nb, db);
+    };
+    if ((long long)(rows / 8) * groups >= 350) launch(k_wgrad_sum<8>, 8);
+    else launch(k_wgrad_sum<4>, 4);
 }
 
 // bpart[block][co] = this block's sum of dY[p][co]; k_wgrad_sum adds the blocks
