@@ -216,8 +216,6 @@ __global__ void __launch_bounds__(TTHREADS) k_conv_fwd_tc(const bf16 *__restrict
     const int r = k / 2, KV = k * k * k, cchunks = Ci / 16;
     const int nkc = KV * cchunks, nkb = (nkc + TKC - 1) / TKC;
 
-    __shared__ __align__(16) float sbias[kMaxCo];
-    const float *sb_ptr = stage_bias<TTHREADS>(sbias, bias, BN);
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tslot)),
                      "r"(tmem_cols));
@@ -328,6 +326,11 @@ __global__ void __launch_bounds__(TTHREADS) k_conv_fwd_tc(const bf16 *__restrict
     }
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
 
+    // the MMAs are done with the stages: the bias goes where the first one was (staged at
+    // the start of the kernel instead, its pointer made the loop above slower: 2 x 9 x 300
+    // positions 160->64 149.9 us against 139.6, 2 x 20 x 40 x 260 96->32 715 against 658)
+    const float *sb_ptr = ok_run ? stage_bias<TTHREADS>(reinterpret_cast<float *>(sm), bias, BN) : nullptr;
+    __syncthreads();
     if (ok_run) {
         // epilogue: warp w owns accumulator rows (TMEM lanes) 32 w .. 32 w + 31
         const long long row = m0 + warp * 32 + lane;

@@ -48,3 +48,30 @@ def test_weight_gradient_sums_are_exact(env, shape, Ci, Co, k, bias):
     assert ws.ws_tc_status() == 0
     assert torch.equal(dw.double(), want + 1.0)
     assert torch.equal(db.double(), want_b + 1.0 if bias else torch.ones_like(want_b))
+
+
+@pytest.mark.parametrize("Ci,Co,k", [(16, 16, 3), (48, 32, 3), (16, 256, 3), (32, 112, 3), (80, 48, 1), (16, 160, 1)])
+@pytest.mark.parametrize("shape", [(1, 1, 1, 1), (1, 2, 3, 260), (2, 3, 5, 7)])
+@pytest.mark.parametrize("f32", [True, False])
+def test_gathered_forward_is_exact(env, shape, Ci, Co, k, f32):
+    """The gathered kernel (lines wider than 254, wide 1x1x1, or on request) with and without
+    bias and ReLU; in BF16 the rounded exact result."""
+    torch, ws = env
+    x, w, b = _ints(torch, shape + (Ci,), Ci), _ints(torch, (Co, k, k, k, Ci), Co), _ints(torch, (Co,), 9, -50, 50)
+    r = k // 2
+    xp = torch.nn.functional.pad(x.double(), (0, 0, r, r, r, r, r, r))
+    N, D, H, W = shape
+    y = sum(xp[:, i:i + D, j:j + H, l:l + W] @ w[:, i, j, l].double().T
+            for i in range(k) for j in range(k) for l in range(k))
+    assert float(y.abs().max()) + 50 < 2 ** 24
+    prev = ws.ws_conv3d_fwd_algo("gather")
+    try:
+        for bias, relu in ((b.float(), True), (None, False), (b.float(), False)):
+            out = torch.full(shape + (Co + 8,), 3.0, dtype=torch.float32 if f32 else torch.bfloat16, device="cuda")
+            ws.ws_conv3d_fwd(x.to(torch.bfloat16), w.to(torch.bfloat16), bias, out[..., :Co], relu)
+            want = y + (b.double() if bias is not None else 0.0)
+            want = (want.clamp(min=0.0) if relu else want).to(out.dtype)
+            assert torch.equal(out[..., :Co], want) and bool((out[..., Co:] == 3.0).all())
+    finally:
+        ws.ws_conv3d_fwd_algo(prev)
+    assert ws.ws_tc_status() == 0
