@@ -1652,7 +1652,7 @@ static bool pers_plan(const ResPlan &res, int Co, ResPlan &p, uint32_t &buf_cols
 // an SM, and a round of resident blocks takes 3000 for the start and the
 // epilogue.  Neither choice changes the order of any sum, so the bits stay.  The search
 // is kept short, because calls of a small grid are bound by their host time (it took
-// 1.2 to 2.7 us, now 0.1 to 0.9).  us per call, before and after: 8^3 128->128 20.6, 16.5; 16^3 96->96 21.7, 13.6;
+// 1.2 to 2.7 us, now 0.1 to 0.5, 1 at 64^3).  us per call, before and after: 8^3 128->128 20.6, 16.5; 16^3 96->96 21.7, 13.6;
 // 224->96 42.9, 26.6; batch 4, 32^3 160->64 114, 94; 64->64 50, 45.  The 10 % are the
 // model's error: at 3 % one sample of 64^3 32->96 goes from 62.6 to 68.0, while 16^3
 // 96->224 at batch 4 goes from 33.4 to 29.2.
@@ -1676,9 +1676,11 @@ static bool small_grid_plan(const Act &a, int Ci, int Co, int sms, ResPlan &plan
     for (int nco : {1, 2, 3, 4, 6, 8}) {
         if (Co % (16 * nco)) continue;
         const int N = Co / nco;
-        // tile counts that hold a line; the last one that matters holds the whole plane
+        // tile counts that hold a line, up to a whole plane or one block per SM (larger
+        // tiles only make that block slower)
         int last_by = 0;
-        for (int want = (a.W + 127) / 128; want * N <= 512 && last_by < ly_max; ++want) {
+        long long m = 2;  // blocks of the busiest SM
+        for (int want = (a.W + 127) / 128; want * N <= 512 && last_by < ly_max && m > 1; ++want) {
             ResPlan p;
             p.by = std::min((128 * want - a.W) / pitch + 1, ly_max);
             p.nyt = (a.H + p.by - 1) / p.by;
@@ -1694,7 +1696,8 @@ static bool small_grid_plan(const Act &a, int Ci, int Co, int sms, ResPlan &plan
             p.a_half = (uint32_t)R * 16u;
             p.stage_bytes = 2 * p.a_half + 18u * (uint32_t)N * 16u;
             p.tx_bytes = 2u * (uint32_t)((p.by + 2) * pitch) * 16u + 18u * (uint32_t)N * 16u;
-            const long long blocks = (long long)a.N * a.D * p.nyt * nco, m = (blocks + sms - 1) / sms;
+            const long long blocks = (long long)a.N * a.D * p.nyt * nco;
+            m = (blocks + sms - 1) / sms;
             // as many resident blocks as the busiest SM has work for, 2 .. 8 stages each
             p.per_sm = (int)std::min<long long>(std::min<long long>(m, 512 / p.cols), 4);
             for (p.stages = 0; p.per_sm >= 1; --p.per_sm) {
