@@ -10,13 +10,16 @@ namespace lbm {
 
 // Occupancy, measured on GB300 (256^3 packed spheres, us per launch).  The
 // collision runs 64-thread blocks, 12 per SM for the FP32 and 16-bit storages
-// (80 registers, no spills of note) and 8 for FP64: FP16 294 against 314 at 11 and
-// 317 at 13 blocks, 310 for 24 blocks of 32 threads; FP32 380 against 397, 423
-// and 402; 6 blocks of 128 threads are 0.5 % slower (rough channel 175.5 against 174.4).
-// The psi pass runs 64-thread blocks, 20 per SM (48 registers, no spills):
-// 16-bit storage 129.7 against 133.7 for 6 blocks of 256 (40 registers) and 131.1
-// for 12 of 128; FP32 176.5 against 179.5 and 178.7; smaller blocks leave no warps
-// waiting for the last of their block.
+// (80 registers; the default update spills 0 to 4 bytes, FP32 with wall slip 48) and
+// 8 for FP64: FP16 294 against 314 at 11 and 317 at 13 blocks, 310 for 24 blocks of
+// 32 threads; FP32 380 against 397, 423 and 402; 6 blocks of 128 threads are 0.5 %
+// slower (rough channel 175.5 against 174.4).
+// The psi pass runs 64-thread blocks, 20 per SM (48 registers): 16-bit storage 129.7
+// against 133.7 for 6 blocks of 256 (40 registers) and 131.1 for 12 of 128; FP32
+// 176.5 against 179.5 and 178.7; smaller blocks leave no warps waiting for the last of
+// their block.  Without wall slip it spills nothing in FP32 and 16 bits and 8 bytes in
+// FP64; with slip it stores 92 bytes (FP32), 164 (16 bits) and 712 (FP64) to local
+// memory, where 6 blocks of 256 threads stored 212, 296 and 940.
 constexpr int kPsiThreads = 64, kPsiBlocks = 20, kCollideThreads = 64;
 template <class S> constexpr int collide_min_blocks() { return sizeof(S) <= 4 ? 12 : 8; }
 

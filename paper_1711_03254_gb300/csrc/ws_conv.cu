@@ -427,7 +427,7 @@ __global__ void __launch_bounds__(kHeadThreads) k_conv1_fwd(const bf16 *__restri
 // bytes without swizzle (two loads and 18) moved twice the TMA rows: 64^3
 // 32->32, batch 4, 441 TFLOP/s against 539.  What bounds it now is the MMA: with the
 // loads left out after the first stages 64^3 32->32 took 106 of its 107 us, some 64
-// clocks per M128 N32 K16 MMA with two blocks per SM, (A + B bytes) / 64 + 20.
+// clocks (43 + 0.65 N) per M128 N32 K16 MMA with two blocks per SM, 16 of them arithmetic.
 //
 // With nco > 1 a block computes Co of the nco x Co output channels (small grids,
 // see small_grid_plan).
@@ -1650,12 +1650,13 @@ static bool pers_plan(const ResPlan &res, int Co, ResPlan &p, uint32_t &buf_cols
 // 105 where one is alone on it, because consecutive MMAs on one accumulator wait
 // for each other; TMA takes 1.5 per 32-byte row; both are shared by the blocks of
 // an SM, and a round of resident blocks takes 3000 for the start and the
-// epilogue.  Neither choice changes the order of any sum, so the bits stay.  The search
-// is kept short, because calls of a small grid are bound by their host time (it took
-// 1.2 to 2.7 us, now 0.1 to 0.5, 1 at 64^3).  us per call, before and after: 8^3 128->128 20.6, 16.5; 16^3 96->96 21.7, 13.6;
-// 224->96 42.9, 26.6; batch 4, 32^3 160->64 114, 94; 64->64 50, 45.  The 10 % are the
-// model's error: at 3 % one sample of 64^3 32->96 goes from 62.6 to 68.0, while 16^3
-// 96->224 at batch 4 goes from 33.4 to 29.2.
+// epilogue.  Neither choice changes the order of any sum, so the bits stay.  The
+// search is kept short, because calls of a small grid are bound by their host time
+// (it took 1.2 to 2.7 us, now 0.1 to 0.5, 1 at 64^3).  us per call, before and after:
+// 8^3 128->128 20.6, 16.5; 16^3 96->96 21.7, 13.6; 224->96 42.9, 26.6; batch 4, 32^3
+// 160->64 114, 94; 64->64 50, 45.  The 10 % are the model's error: at 3 % one sample
+// of 64^3 32->96 goes from 62.6 to 68.0, while 16^3 96->224 at batch 4 goes from 33.4
+// to 29.2.
 static double grid_cost(const Act &a, int Ci, int N, int nco, const ResPlan &p, int sms) {
     const long long blocks = (long long)a.N * a.D * p.nyt * nco;
     const long long m = (blocks + sms - 1) / sms;  // blocks of the busiest SM

@@ -1,14 +1,19 @@
 """The persistent compact update (LBM_KERNEL_PERSISTENT): n updates of the
-compact two-pass update in one cooperative launch with grid-wide barriers.
+compact two-pass update in one launch.  FP64, and instances of more than 8192
+non-solid cells, run one cooperative launch with grid-wide barriers; smaller
+instances in the other storages stay in the shared memory of a thread-block
+cluster each (which most shapes here do; test_gpu_persist_grid.py holds the
+larger ones).
 
-It runs the same per-cell code as the two-launch compact update (loads of data
-written in the same launch go through L2), so the states must agree bit for
-bit: fields and distributions, after any number of updates, over ragged grids,
-batches, both equilibria, the third-order regularisation, every wall model and
-INLET/OUTLET planes; in the steady-state loop too.  The failure path: with a
-barrier that waits for an arrival that never comes, every block gives up
-after the bound and the host reports LBM_ERR_TIMEOUT, and the context stays
-usable.  A timing comparison on batched small instances is printed."""
+Both run the same per-cell code as the two-launch compact update (with the
+barriers, loads of data written in the same launch go through L2), so the states
+must agree bit for bit: fields and distributions, after any number of updates,
+over ragged grids, batches, both equilibria, the third-order regularisation,
+every wall model and INLET/OUTLET planes; in the steady-state loop too.  The
+failure path: with a barrier that waits for an arrival that never comes, every
+block gives up after the bound and the host reports LBM_ERR_TIMEOUT, and the
+context stays usable.  A timing comparison on batched small instances is
+printed."""
 import time
 
 import numpy as np
