@@ -32,6 +32,7 @@ import argparse
 import hashlib
 import json
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -91,7 +92,8 @@ def alg_bytes_per_cell(part: str, precision: str) -> int:
 # DRAM traffic of the dominant kernel from one ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum of a launch / its fluid cells),
 # keyed by kernel/precision/workload, with the hash of the source files the
-# kernel is built from at the time of the capture; any change of them voids it.
+# kernel is built from at the time of the capture (sources_hash: code without
+# comments); any change of their code voids it.
 COMPACT_SOURCES = ["lbm_types.h", "lbm_device.cuh", "lbm_pair2.cuh", "lbm_compact.cuh", "lbm_compact_update.cuh"]
 DENSE_SOURCES = ["lbm_types.h", "lbm_device.cuh", "lbm_twopass.cuh"]
 NCU_TRAFFIC = {
@@ -101,22 +103,27 @@ NCU_TRAFFIC = {
                                 "how": "ncu --set full, one launch at 128^3, scaled by non-solid cells"},
     # the benchmark itself (256^3, 6,710,661 non-solid cells), one launch each,
     # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum:
-    #   k_collide_c2: 649,660,672 B read + 497,568,000 B written = 171.0 B per cell
-    #   k_psi_c:      595,477,504 B read +  50,510,080 B written =  96.3 B per cell
-    "k_collide_c2/fp16s/spheres": {"bytes_per_fluid_cell": 170.96, "src": "856ecc299163ec5a",
-                                   "files": COMPACT_SOURCES, "step_bytes_per_fluid_cell": 170.96 + 96.26,
+    #   k_collide_c2: 649.63 MB read + 491.07 MB written = 169.98 B per cell
+    #   k_psi_c:      595.47 MB read +  50.26 MB written =  96.23 B per cell
+    "k_collide_c2/fp16s/spheres": {"bytes_per_fluid_cell": 169.98, "src": "da84f6b5868da85c",
+                                   "files": COMPACT_SOURCES, "step_bytes_per_fluid_cell": 169.98 + 96.23,
                                    "how": "ncu dram__bytes_read.sum + dram__bytes_write.sum, one launch at 256^3"},
 }
 # FP64 mode is bound by the FP64 pipe.  Executed FP64 flops per non-solid cell
 # (DADD + DMUL + 2 DFMA from ncu, 128^3 packed spheres, eq_order 0) and the
 # FP64 peak: 2 DFMA per clock per SM (152 SMs, 2.07 GHz) = 1.26 TFLOP/s.
-# (Counted on sources 4ac21a08ce947105; the next change of these files touched
-# only the psi pass, so the FP64 update's code is the one counted.)
-FP64_FLOPS = {"k_collide_c": {"flops_per_fluid_cell": 813.7, "src": "1f62a0de098d92be", "files": COMPACT_SOURCES}}
+FP64_FLOPS = {"k_collide_c": {"flops_per_fluid_cell": 814.7, "src": "da84f6b5868da85c", "files": COMPACT_SOURCES}}
 FP64_PEAK_TFLOPS = 2 * 2 * 152 * 2.07e9 / 1e12
 
 
 E2E_SAMPLES = 3
+
+
+def code_only(text: str) -> str:
+    """C++ source without comments, one space for any run of white space (the
+    kernels' sources hold no string with a comment mark in it)."""
+    text = re.sub(r"/\*.*?\*/", " ", text, flags=re.S)
+    return " ".join(re.sub(r"//[^\n]*", " ", text).split())
 
 
 def sources_hash(files=COMPACT_SOURCES) -> str:
@@ -124,7 +131,7 @@ def sources_hash(files=COMPACT_SOURCES) -> str:
     for s in files:
         p = os.path.join(ROOT, "paper_1711_03254_gb300", "csrc", s)
         if os.path.exists(p):
-            h.update(open(p, "rb").read())
+            h.update(code_only(open(p).read()).encode())
     return h.hexdigest()[:16]
 
 
