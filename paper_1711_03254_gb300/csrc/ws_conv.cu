@@ -1409,7 +1409,7 @@ __global__ void __launch_bounds__(32 * kSumLanes) k_wgrad_sum(const float *__res
 // 8 rows a block where that makes 350 blocks or more, else 4 with twice the chunks in
 // flight: a block waits for its chunks one after the other, and few blocks leave SMs
 // idle (weight gradient of 32^3 16->16 22.9 us with 8 rows, 16.9 with 4; 64^3 32->32 43.4
-// and 37.4; the other way round 32^3 128->128 51.6 and 54.6).
+// and 37.4; with more blocks 8 rows are faster: 32^3 128->128 51.6 and 54.6).
 static void launch_wgrad_sum(const float *part, int nk, int rows_pad, int rows, int Co, int KV, int Ci, float *dw,
                              const float *bpart, int nb, float *db, cudaStream_t s) {
     const unsigned groups = (unsigned)((Co + 31) / 32);
